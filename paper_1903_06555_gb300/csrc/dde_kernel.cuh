@@ -225,15 +225,17 @@ template <typename T, typename C>
 __global__ void __launch_bounds__(VisLaunch<T>::threads, VisLaunch<T>::min_blocks)
     dde_box_kernel(const VisRec<T>* __restrict__ recs, int64_t n, C* __restrict__ boxes,
                    int jmax, QuadParams q, unsigned long long* head,
-                   unsigned long long* stats, int batch) {
+                   unsigned long long* stats, int batch, RecordList list) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   NodeVal<T>* sh = reinterpret_cast<NodeVal<T>*>(smem_raw) + warp * kNodeBatch;
   unsigned long long my_bad = 0, my_nodes = 0;
+  n = list.count(n);
   WarpQueue wq;
   unsigned long long i;
   while (wq.take(head, static_cast<unsigned long long>(batch), n, lane, i)) {
+    i = list.record(i);
     const VisRec<T> r = recs[i];
     const int Jw = r.jw, half = Jw / 2, ntap = Jw * Jw;
     C* box = boxes + static_cast<int64_t>(i) * jmax * jmax;
@@ -289,7 +291,8 @@ __global__ void __launch_bounds__(VisLaunch<T>::threads, VisLaunch<T>::min_block
 template <typename T, typename C>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) dde_box_radial_kernel(
     const VisRec<T>* __restrict__ recs, int64_t n, C* __restrict__ boxes, int jmax, QuadParams q,
-    RadialView<T> rv, unsigned long long* head, unsigned long long* stats, int batch) {
+    RadialView<T> rv, unsigned long long* head, unsigned long long* stats, int batch,
+    RecordList list) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -297,9 +300,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) dde_box_radial_ke
   C* ser = reinterpret_cast<C*>(smem_raw + (blockDim.x >> 5) * kNodeBatch * sizeof(NodeVal<T>)) +
            warp * rv.buf;
   unsigned long long my_bad = 0, my_nodes = 0;
+  n = list.count(n);
   WarpQueue wq;
   unsigned long long i;
   while (wq.take(head, static_cast<unsigned long long>(batch), n, lane, i)) {
+    i = list.record(i);
     const VisRec<T> r = recs[i];
     const int Jw = r.jw, half = Jw / 2, ntap = Jw * Jw;
     C* box = boxes + static_cast<int64_t>(i) * jmax * jmax;

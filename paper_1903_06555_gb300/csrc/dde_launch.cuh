@@ -46,6 +46,7 @@ int launch_dde_two_pass(Plan& p, const VisRec<T>* recs, int64_t b0, int64_t nk, 
   // pass 1: the plain kernel's block shape and shared memory (limits set
   // to one value for all plans, so concurrent launchers agree)
   const bool radial = p.d.kernel_mode == PHI_KERNEL_RADIAL;
+  const bool series = p.series_stride > 0;
   constexpr int box_threads = VisLaunch<T>::threads;
   const size_t box_smem = radial ? radial_smem<T, C>(p)
                                  : (box_threads / 32) * kNodeBatch * sizeof(NodeVal<T>);
@@ -85,14 +86,28 @@ int launch_dde_two_pass(Plan& p, const VisRec<T>* recs, int64_t b0, int64_t nk, 
       st = PHI_ERR_CUDA;
       break;
     }
+    // the boxes at the samples in rho, then the records those left
+    RecordList list{nullptr, nullptr};
+    unsigned long long* box_head = head;
+    int batch = queue_batch(n, box_blocks * (box_threads / 32));
+    if (series) {
+      box_head = p.retry_counters + 2 * g + 1;
+      if (cudaMemsetAsync(p.retry_counters + 2 * g, 0, 2 * sizeof(unsigned long long), s) !=
+              cudaSuccess ||
+          launch_box_series<T, C>(p, g, recs + c0, n, boxes, jmax, s) != PHI_OK) {
+        st = PHI_ERR_CUDA;
+        break;
+      }
+      list = RecordList{p.retry, p.retry_counters + 2 * g};
+      batch = 1;
+    }
     if (radial)
       dde_box_radial_kernel<T, C><<<box_blocks, box_threads, box_smem, s>>>(
-          recs + c0, n, boxes, jmax, p.quad(), radial_view<T, C>(p), head, p.counters + p.K,
-          queue_batch(n, box_blocks * (box_threads / 32)));
+          recs + c0, n, boxes, jmax, p.quad(), radial_view<T, C>(p), box_head, p.counters + p.K,
+          batch, list);
     else
       dde_box_kernel<T, C><<<box_blocks, box_threads, box_smem, s>>>(
-          recs + c0, n, boxes, jmax, p.quad(), head, p.counters + p.K,
-          queue_batch(n, box_blocks * (box_threads / 32)));
+          recs + c0, n, boxes, jmax, p.quad(), box_head, p.counters + p.K, batch, list);
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemsetAsync(head, 0, sizeof(unsigned long long), s) != cudaSuccess) {
       st = PHI_ERR_CUDA;

@@ -112,6 +112,24 @@ struct RadialView {
   int buf;
 };
 
+// Kernel-side view of the sampled quadrature (series_kernel.cuh): J0 at the
+// samples rho_i = i / inv_delta for every node of panel counts up to
+// max_panels, the node table's 1 - n as two floats (FP32), the list of the
+// records left to the per-tap kernels and its length.
+template <typename T>
+struct SeriesView {
+  const T* j0;
+  const float2* omn2;
+  int stride;          // samples per table row
+  int max_panels, max_intervals;
+  int support;         // J
+  T inv_delta;         // 4 R
+  float inv_delta_f, inv_cycles;
+  T tol;
+  uint32_t* retry;
+  unsigned long long* n_retry;
+};
+
 // Deterministic gridding target (grid_deterministic = 1): per grid cell two
 // int64 (re, im) holding the cell's sum in units of 2^-exp[0], so that the
 // sum does not depend on the order of its additions; exp[1] != 0 marks a
@@ -143,7 +161,7 @@ struct Plan {
   phi_plan_desc d;
   int N = 0, npad = 0, K = 0;
   double dl = 0, du = 0, R = 0, beta = 0, i0beta = 0, l_win = 0, n_win = 0, c_support = 0;
-  double cycles_per_panel = 0;
+  double cycles_per_panel = 0, auto_cycles_per_panel = 0;
   int64_t M = 0, n_kept = 0, n_dropped = 0;
   int kmeans_sweeps = 0;
   int max_jw = 0;
@@ -170,8 +188,11 @@ struct Plan {
   cufftHandle fft_batch = 0;            // `group` transforms in one call
   bool fft_batch_ok = false;
   // [0..K) work heads, [K] unconverged taps, [K+1] taps, [K+2] wkernel misses,
-  // [K+3] tap-node evaluations
+  // [K+3] tap-node evaluations; retry_counters[2 g], [2 g + 1], g < K: length
+  // of group g's retry list and the head of the queue that takes it, just
+  // before the work heads so that one memset clears both
   unsigned long long* counters = nullptr;
+  unsigned long long* retry_counters = nullptr;
   // per-stage timing
   bool timing = false;
   std::vector<cudaEvent_t> ev_pool;
@@ -206,6 +227,14 @@ struct Plan {
   void* radial_tab = nullptr;
   double radial_L = 0;
   int radial_buf = 0;
+  // sampled quadrature (series_kernel.cuh; PHI_KERNEL_QUADRATURE and
+  // PHI_KERNEL_RADIAL): J0 table, 1 - n in two floats, retry list of the kept
+  // records; series_stride = 0: not in use
+  void* series_j0 = nullptr;
+  float2* series_omn2 = nullptr;
+  uint32_t* retry = nullptr;
+  int series_stride = 0, series_max_panels = 0, series_max_intervals = 0;
+  float series_inv_cycles = 0;
   // deterministic gridding (grid_deterministic = 1): fixed-point sums of the
   // group's grids (group * Npad^2 * 2 int64), the largest |W_i y_i| term
   // factor of a call (double bits), the exponent and non-finite flag, and
@@ -273,6 +302,7 @@ int launch_node_tables(Plan& p, cudaStream_t s);
 int launch_pixel_tables(Plan& p, cudaStream_t s);
 int build_kernel_table(Plan& p, cudaStream_t s);
 int build_radial_tables(Plan& p, cudaStream_t s);
+int build_series_tables(Plan& p, cudaStream_t s);
 int compute_kernel_bound(Plan& p, double* scratch, cudaStream_t s);  // scratch: kMaxPanels doubles
 
 }  // namespace phi

@@ -898,6 +898,19 @@ struct WarpQueue {
   }
 };
 
+// The records a per-tap kernel takes: [0, n), or, with a list, the records
+// the list names (its length known on the device only).
+struct RecordList {
+  const uint32_t* index;
+  const unsigned long long* n;
+  __device__ __forceinline__ int64_t count(int64_t all) const {
+    return index ? static_cast<int64_t>(*n) : all;
+  }
+  __device__ __forceinline__ unsigned long long record(unsigned long long i) const {
+    return index ? index[i] : i;
+  }
+};
+
 // The value a gridded visibility spreads: W_i y_i, conjugated back if folded.
 template <typename T, typename C>
 __device__ __forceinline__ C load_visibility(const C* __restrict__ vis_in, uint32_t pm, T weight) {
@@ -988,16 +1001,18 @@ __global__ void __launch_bounds__(VisLaunch<T>::threads, VisLaunch<T>::min_block
     vis_kernel(const VisRec<T>* __restrict__ recs, const uint32_t* __restrict__ perm, int64_t n,
                const C* __restrict__ grid_in, C* grid_out, const C* __restrict__ vis_in,
                C* __restrict__ vis_out, QuadParams q, const int32_t* __restrict__ stack_slot,
-               unsigned long long* head, unsigned long long* stats, int batch) {
+               unsigned long long* head, unsigned long long* stats, int batch, RecordList list) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   NodeVal<T>* sh = reinterpret_cast<NodeVal<T>*>(smem_raw) + warp * kNodeBatch;
   unsigned long long my_bad = 0, my_taps = 0, my_nodes = 0;
   const int npad = q.npad;
+  n = list.count(n);
   WarpQueue wq;
   unsigned long long i;
   while (wq.take(head, static_cast<unsigned long long>(batch), n, lane, i)) {
+    i = list.record(i);
     const VisRec<T> r = recs[i];
     const int Jw = r.jw;
     // the grid of this visibility's stack within the resident group
@@ -1608,7 +1623,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) vis_radial_kernel
     const C* __restrict__ grid_in, C* grid_out, const C* __restrict__ vis_in,
     C* __restrict__ vis_out, QuadParams q, RadialView<T> rv,
     const int32_t* __restrict__ stack_slot, unsigned long long* head,
-    unsigned long long* stats, int batch) {
+    unsigned long long* stats, int batch, RecordList list) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -1617,9 +1632,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) vis_radial_kernel
            warp * rv.buf;
   unsigned long long my_bad = 0, my_taps = 0, my_nodes = 0;
   const int npad = q.npad;
+  n = list.count(n);
   WarpQueue wq;
   unsigned long long i;
   while (wq.take(head, static_cast<unsigned long long>(batch), n, lane, i)) {
+    i = list.record(i);
     const VisRec<T> r = recs[i];
     const int Jw = r.jw;
     const int64_t gbase = static_cast<int64_t>(stack_slot[r.stack]) * npad * npad;
@@ -1668,6 +1685,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) vis_radial_kernel
   }
   flush_counts(stats, my_bad, my_taps, my_nodes, lane);
 }
+
+// The quadrature at samples in rho: vis_series_kernel, dde_box_series_kernel
+#include "series_kernel.cuh"
 
 // Direction-dependent effects (Sec. 5.2): vis_dde_kernel
 #include "dde_kernel.cuh"
@@ -1895,7 +1915,8 @@ struct DdeArgs {
   int jd;
 };
 
-// dde_warp_smem, launch_dde
+// launch_series, dde_warp_smem, launch_dde
+#include "series_launch.cuh"
 #include "dde_launch.cuh"
 
 template <typename T, typename C, bool kGrid>
@@ -1925,6 +1946,20 @@ int launch_group_kernel(Plan& p, int g, const C* grids_in, C* grids_out, const C
   const int64_t nk = p.stack_off[p.group_stacks[s1 - 1] + 1] - b0;
   if (nk == 0) return PHI_OK;
   const VisRec<T>* recs = static_cast<const VisRec<T>*>(p.recs) + b0;
+  // the sampled quadrature whenever the plan has its tables (both modes: it is
+  // 6 times the per-tap kernel and 2-5 times the radial series at every
+  // support measured, 4 to 64); the per-tap kernel then takes the list of
+  // those it left (as a rule none: the launch finds it empty, 2.5 us)
+  RecordList list{nullptr, nullptr};
+  unsigned long long* head = p.counters + g;
+  int batch = 0;
+  if (p.series_stride > 0) {
+    PHI_TRY_ST((launch_series<T, C, kGrid>(p, g, recs, b0, nk, grids_in, grids_out, vis_in,
+                                           vis_out, s)));
+    list = RecordList{p.retry, p.retry_counters + 2 * g};
+    head = p.retry_counters + 2 * g + 1;
+    batch = 1;
+  }
   if (p.d.kernel_mode == PHI_KERNEL_RADIAL) {
     const size_t smem = radial_smem<T, C>(p);
     int per_sm = 0;
@@ -1935,8 +1970,8 @@ int launch_group_kernel(Plan& p, int g, const C* grids_in, C* grids_out, const C
     const int blocks = per_sm * p.num_sms;
     vis_radial_kernel<T, C, kGrid><<<blocks, kVisThreads, smem, s>>>(
         recs, p.perm + b0, nk, grids_in, grids_out, vis_in, vis_out, p.quad(),
-        radial_view<T, C>(p), p.stack_slot_dev, p.counters + g, p.counters + p.K,
-        queue_batch(nk, blocks * (kVisThreads / 32)));
+        radial_view<T, C>(p), p.stack_slot_dev, head, p.counters + p.K,
+        batch ? batch : queue_batch(nk, blocks * (kVisThreads / 32)), list);
   } else if (p.d.kernel_mode == PHI_KERNEL_TABLE) {
     const int blocks = p.num_sms * 8;
     vis_table_kernel<T, C, kGrid><<<blocks, kVisThreads, 0, s>>>(
@@ -1949,7 +1984,7 @@ int launch_group_kernel(Plan& p, int g, const C* grids_in, C* grids_out, const C
     const int blocks = blocks_for_vis<T, C>(p, smem);
     vis_kernel<T, C, kGrid><<<blocks, threads, smem, s>>>(
         recs, p.perm + b0, nk, grids_in, grids_out, vis_in, vis_out, p.quad(), p.stack_slot_dev,
-        p.counters + g, p.counters + p.K, queue_batch(nk, blocks * (threads / 32)));
+        head, p.counters + p.K, batch ? batch : queue_batch(nk, blocks * (threads / 32)), list);
   }
   PHI_CUDA_TRY(cudaGetLastError());
   return PHI_OK;
@@ -1959,7 +1994,7 @@ template <typename T, typename C>
 int run_degrid(Plan& p, const T* x, C* y, cudaStream_t s, const DdeArgs* dde = nullptr) {
   long ev = timer_begin(p, s);
   PHI_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(C) * (size_t)p.M, s));
-  PHI_CUDA_TRY(cudaMemsetAsync(p.counters, 0, sizeof(unsigned long long) * p.K, s));
+  PHI_CUDA_TRY(cudaMemsetAsync(p.retry_counters, 0, sizeof(unsigned long long) * 3 * p.K, s));
   timer_end(p, ev, PHI_STAGE_CLEAR, s);
   C* grids = static_cast<C*>(p.grid);
   const int ngroups = static_cast<int>(p.group_off.size()) - 1;
@@ -2018,7 +2053,7 @@ int fixed_prepare(Plan& p, int g, const C* y, const DdeArgs* dde, cudaStream_t s
 
 template <typename T, typename C>
 int run_grid(Plan& p, const C* y, T* x, cudaStream_t s, const DdeArgs* dde = nullptr) {
-  PHI_CUDA_TRY(cudaMemsetAsync(p.counters, 0, sizeof(unsigned long long) * p.K, s));
+  PHI_CUDA_TRY(cudaMemsetAsync(p.retry_counters, 0, sizeof(unsigned long long) * 3 * p.K, s));
   C* grids = static_cast<C*>(p.grid);
   const int64_t plane = static_cast<int64_t>(p.npad) * p.npad;
   const int ngroups = static_cast<int>(p.group_off.size()) - 1;
@@ -2086,6 +2121,11 @@ int build_radial_tables(Plan& p, cudaStream_t s) {
   return build_radial_tables_t<float, float2>(p, s);
 }
 
+int build_series_tables(Plan& p, cudaStream_t s) {
+  if (p.d.precision == PHI_F64) return build_series_tables_t<double, double2>(p, s);
+  return build_series_tables_t<float, float2>(p, s);
+}
+
 int compute_kernel_bound(Plan& p, double* scratch, cudaStream_t s) {
   const int blocks = (kMaxPanels + 127) / 128;
   if (p.d.precision == PHI_F64)
@@ -2119,6 +2159,15 @@ void timer_end(Plan& p, long idx, int stage, cudaStream_t s) {
   if (idx < 0) return;
   if (cudaEventRecord(p.ev_pool[idx + 1], s) != cudaSuccess) return;
   p.ev_pending.emplace_back(stage, static_cast<size_t>(idx));
+}
+
+template <typename T, typename C>
+cudaError_t set_series_smem(int bytes) {
+  const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(vis_series_kernel<T, C, false>, a, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(vis_series_kernel<T, C, true>, a, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(dde_box_series_kernel<T, C>, a, bytes);
+  return e;
 }
 
 template <typename T, typename C>
@@ -2183,6 +2232,8 @@ int set_kernel_smem_limits() {
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
   PHI_CUDA_TRY(cudaFuncSetAttribute(vis_radial_kernel<double, double2, true>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+  PHI_CUDA_TRY((set_series_smem<float, float2>(optin)));
+  PHI_CUDA_TRY((set_series_smem<double, double2>(optin)));
   PHI_CUDA_TRY((set_dde_smem<float, float2>(optin)));
   PHI_CUDA_TRY((set_dde_smem<double, double2>(optin)));
   // table staging: patch and row sizes depend on the plan; the attribute is

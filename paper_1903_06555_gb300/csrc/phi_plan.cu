@@ -332,7 +332,10 @@ void free_plan(Plan* p) {
   cudaFree(p->tap_off);
   cudaFree(p->radial_tab);
   cudaFree(p->grid);
-  cudaFree(p->counters);
+  cudaFree(p->retry_counters);
+  cudaFree(p->series_j0);
+  cudaFree(p->series_omn2);
+  cudaFree(p->retry);
   cudaFree(p->table);
   cudaFree(p->item_start);
   cudaFree(p->item_key);
@@ -456,9 +459,8 @@ int build(Plan& p, const double* uvw, const double* weights, int64_t M, cudaStre
   // Gauss-Kronrod 15/31 panels of about 6 integrand cycles at the paper's
   // tolerance 1e-6, narrowing slowly with the tolerance (3.4 cycles at 1e-12):
   // the widths that gave the fewest tap-nodes, refinements included
-  p.cycles_per_panel = d.cycles_per_panel > 0.0
-                           ? d.cycles_per_panel
-                           : std::min(8.0, std::max(1.0, 6.0 * std::pow(tol / 1e-6, 1.0 / 24.0)));
+  p.auto_cycles_per_panel = std::min(8.0, std::max(1.0, 6.0 * std::pow(tol / 1e-6, 1.0 / 24.0)));
+  p.cycles_per_panel = d.cycles_per_panel > 0.0 ? d.cycles_per_panel : p.auto_cycles_per_panel;
 
   int dev = 0;
   PHI_CUDA_TRY(cudaGetDevice(&dev));
@@ -470,8 +472,9 @@ int build(Plan& p, const double* uvw, const double* weights, int64_t M, cudaStre
   p.stack_off.assign(K + 1, 0);
   p.stack_jw.assign(K, 0);
   p.stack_maxabs.assign(K, 0.0);
-  PHI_CUDA_TRY(owned_alloc(p, &p.counters, static_cast<size_t>(K) + 4));
-  PHI_CUDA_TRY(cudaMemsetAsync(p.counters, 0, sizeof(unsigned long long) * (K + 4), s));
+  PHI_CUDA_TRY(owned_alloc(p, &p.retry_counters, 3 * static_cast<size_t>(K) + 4));
+  p.counters = p.retry_counters + 2 * K;
+  PHI_CUDA_TRY(cudaMemsetAsync(p.retry_counters, 0, sizeof(unsigned long long) * (3 * K + 4), s));
 
   Scratch tmp;
   const int nblk = std::max(1, std::min<int>(p.num_sms * 4,
@@ -806,6 +809,7 @@ int build(Plan& p, const double* uvw, const double* weights, int64_t M, cudaStre
     PHI_TRY(build_kernel_table(p, s));
   }
   if (d.kernel_mode == PHI_KERNEL_RADIAL) PHI_TRY(build_radial_tables(p, s));
+  if (d.kernel_mode != PHI_KERNEL_TABLE) PHI_TRY(build_series_tables(p, s));
   if (cufftCreate(&p.fft) != CUFFT_SUCCESS) return PHI_ERR_CUDA;
   p.fft_ok = true;
   size_t work = 0;

@@ -1,0 +1,137 @@
+// Host side of the sampled quadrature (series_kernel.cuh).  Not a standalone
+// header: phi_ops.cu includes it inside its host-side anonymous namespace,
+// after queue_batch.
+#pragma once
+
+template <typename T, typename C>
+SeriesView<T> series_view(const Plan& p, int g) {
+  SeriesView<T> v;
+  v.j0 = static_cast<const T*>(p.series_j0);
+  v.omn2 = p.series_omn2;
+  v.stride = p.series_stride;
+  v.max_panels = p.series_max_panels;
+  v.max_intervals = p.series_max_intervals;
+  v.support = p.d.support;
+  v.inv_delta = static_cast<T>(4.0 * p.R);
+  v.inv_delta_f = static_cast<float>(4.0 * p.R);
+  v.inv_cycles = p.series_inv_cycles;
+  v.tol = static_cast<T>(p.d.quad_abs_tol);
+  v.retry = p.retry;
+  v.n_retry = p.retry_counters + 2 * g;
+  return v;
+}
+
+// The smallest absolute tolerance the estimate can meet: FP32 panel sums
+// carry about 1e-7 of rounding, FP64 ones 1e-15.
+template <typename T>
+constexpr double series_least_tol() { return sizeof(T) == 4 ? 2.5e-7 : 1e-14; }
+
+// J0 table for the panel counts and supports of this plan.  Panels no wider
+// than the automatic width, so that a plan with wide panels of its own still
+// passes the estimate.
+template <typename T, typename C>
+int build_series_tables_t(Plan& p, cudaStream_t s) {
+  if (p.n_kept == 0 || p.d.quad_abs_tol < series_least_tol<T>()) return PHI_OK;
+  p.series_inv_cycles =
+      static_cast<float>(1.0 / std::min(p.cycles_per_panel, p.auto_cycles_per_panel));
+  int panels = 1, intervals = 1;
+  const float inv_delta = static_cast<float>(4.0 * p.R);
+  for (int k = 0; k < p.K; ++k) {
+    if (p.stack_jw[k] == 0) continue;
+    intervals = std::max(intervals, series_intervals(p.stack_jw[k], inv_delta));
+    panels = std::max(panels, series_panels(p.stack_jw[k], p.d.support, static_cast<float>(p.R),
+                                            static_cast<float>(p.c_support), p.series_inv_cycles,
+                                            static_cast<float>(p.stack_maxabs[k])));
+  }
+  p.series_max_panels = std::min(panels, kSeriesMaxPanels);
+  p.series_max_intervals = std::min(intervals, kSeriesMaxSamples - SeriesN<T>::half);
+  const int stride = (p.series_max_intervals + SeriesN<T>::half + 31) / 32 * 32;
+  const int64_t rows = panel_table_offset(p.series_max_panels + 1);
+  void* raw = nullptr;
+  PHI_CUDA_TRY(cudaMalloc(&raw, sizeof(T) * rows * stride));
+  p.series_j0 = raw;
+  p.device_bytes += static_cast<int64_t>(sizeof(T) * rows * stride);
+  if (sizeof(T) == 4) {
+    PHI_CUDA_TRY(cudaMalloc(&raw, sizeof(float2) * rows));
+    p.series_omn2 = static_cast<float2*>(raw);
+    p.device_bytes += static_cast<int64_t>(sizeof(float2) * rows);
+  }
+  PHI_CUDA_TRY(cudaMalloc(&raw, sizeof(uint32_t) * p.n_kept));
+  p.retry = static_cast<uint32_t*>(raw);
+  p.device_bytes += static_cast<int64_t>(sizeof(uint32_t) * p.n_kept);
+  const int blocks =
+      static_cast<int>(std::min<int64_t>((rows * stride + 255) / 256, p.num_sms * 8));
+  series_table_kernel<T><<<blocks, 256, 0, s>>>(p.node_omn, rows, stride,
+                                                static_cast<T*>(p.series_j0), p.series_omn2);
+  PHI_CUDA_TRY(cudaGetLastError());
+  p.series_stride = stride;
+  return PHI_OK;
+}
+
+// Block shape: as many warps per block (at most 8) as keep the most warps
+// resident, each with its own samples and polynomials.
+struct SeriesShape {
+  int warps = 0, blocks = 0, batch = 1;
+  size_t smem = 0;
+};
+template <typename T, typename C, typename K>
+int series_shape(const Plan& p, K kernel, int64_t n, SeriesShape& sh) {
+  const size_t per_warp = series_warp_bytes<T>(p.series_stride, p.series_max_intervals);
+  int dev = 0, optin = 0, per_sm_smem = 0, reserved = 0;
+  PHI_CUDA_TRY(cudaGetDevice(&dev));
+  PHI_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  PHI_CUDA_TRY(cudaDeviceGetAttribute(&per_sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor,
+                                      dev));
+  PHI_CUDA_TRY(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev));
+  int best = 0;
+  for (int w = 1; w <= kVisThreads / 32; ++w) {
+    const size_t blk = per_warp * w;
+    if (blk > static_cast<size_t>(optin)) break;
+    const int resident = w * static_cast<int>(per_sm_smem / (blk + reserved));
+    if (resident >= best) {
+      best = resident;
+      sh.warps = w;
+    }
+  }
+  if (sh.warps == 0) return PHI_ERR_SUPPORT;   // not reached: one warp takes 31 KB at most
+  sh.smem = per_warp * sh.warps;
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * sh.warps, sh.smem) !=
+          cudaSuccess ||
+      per_sm < 1)
+    per_sm = 1;
+  sh.blocks = per_sm * p.num_sms;
+  // pairs are taken within a batch: batches of an even number once there are
+  // several visibilities to a warp, single visibilities before that
+  const int64_t warps = static_cast<int64_t>(sh.blocks) * sh.warps;
+  sh.batch = queue_batch(n, warps);
+  if (sh.batch < 2 && n >= 4 * warps) sh.batch = 2;
+  if (sh.batch > 1) sh.batch &= ~1;
+  return PHI_OK;
+}
+
+// The fused kernel over nk records (the plan's records from b0 on).
+template <typename T, typename C, bool kGrid>
+int launch_series(Plan& p, int g, const VisRec<T>* recs, int64_t b0, int64_t nk, const C* grids_in,
+                  C* grids_out, const C* vis_in, C* vis_out, cudaStream_t s) {
+  SeriesShape sh;
+  PHI_TRY_ST((series_shape<T, C>(p, vis_series_kernel<T, C, kGrid>, nk, sh)));
+  vis_series_kernel<T, C, kGrid><<<sh.blocks, 32 * sh.warps, sh.smem, s>>>(
+      recs, p.perm + b0, nk, grids_in, grids_out, vis_in, vis_out, p.quad(),
+      series_view<T, C>(p, g), p.stack_slot_dev, p.counters + g, p.counters + p.K, sh.batch);
+  PHI_CUDA_TRY(cudaGetLastError());
+  return PHI_OK;
+}
+
+// The DDE convolution's boxes of n records.
+template <typename T, typename C>
+int launch_box_series(Plan& p, int g, const VisRec<T>* recs, int64_t n, C* boxes, int jmax,
+                      cudaStream_t s) {
+  SeriesShape sh;
+  PHI_TRY_ST((series_shape<T, C>(p, dde_box_series_kernel<T, C>, n, sh)));
+  dde_box_series_kernel<T, C><<<sh.blocks, 32 * sh.warps, sh.smem, s>>>(
+      recs, n, boxes, jmax, p.quad(), series_view<T, C>(p, g), p.counters + g, p.counters + p.K,
+      sh.batch);
+  PHI_CUDA_TRY(cudaGetLastError());
+  return PHI_OK;
+}
