@@ -114,16 +114,18 @@ struct RadialView {
 
 // Kernel-side view of the sampled quadrature (series_kernel.cuh): J0 at the
 // samples rho_i = i / inv_delta for every node of panel counts up to
-// max_panels, the node table's 1 - n as two floats (FP32), the list of the
-// records left to the per-tap kernels and its length.
+// max_panels (FP64 a table of values, FP32 matrix tiles with a node table),
+// the list of the records left to the per-tap kernels and its length.
 template <typename T>
 struct SeriesView {
-  const T* j0;
-  const float2* omn2;
-  int stride;          // samples per table row
+  const double* j0;        // FP64: [node][stride]
+  const uint4* tiles_a;    // FP32: [panel][tile][step][hi, lo][lane]
+  const float4* nodes;     // FP32: [panel][step][16]
+  int stride;              // samples the tables hold
+  int tiles;               // stride / 16
   int max_panels, max_intervals;
-  int support;         // J
-  T inv_delta;         // 4 R
+  int support;             // J
+  T inv_delta;             // 4 R
   float inv_delta_f, inv_cycles;
   T tol;
   uint32_t* retry;
@@ -228,10 +230,10 @@ struct Plan {
   double radial_L = 0;
   int radial_buf = 0;
   // sampled quadrature (series_kernel.cuh; PHI_KERNEL_QUADRATURE and
-  // PHI_KERNEL_RADIAL): J0 table, 1 - n in two floats, retry list of the kept
+  // PHI_KERNEL_RADIAL): J0 table, node table (FP32), retry list of the kept
   // records; series_stride = 0: not in use
   void* series_j0 = nullptr;
-  float2* series_omn2 = nullptr;
+  float4* series_nodes = nullptr;
   uint32_t* retry = nullptr;
   int series_stride = 0, series_max_panels = 0, series_max_intervals = 0;
   float series_inv_cycles = 0;

@@ -19,6 +19,7 @@
 // max_refine times); taps still above tolerance are counted.  The degridder
 // and the gridder run this identical routine, so [GC] and its conjugate
 // transpose pair exactly.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>

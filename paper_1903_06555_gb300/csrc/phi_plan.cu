@@ -334,7 +334,7 @@ void free_plan(Plan* p) {
   cudaFree(p->grid);
   cudaFree(p->retry_counters);
   cudaFree(p->series_j0);
-  cudaFree(p->series_omn2);
+  cudaFree(p->series_nodes);
   cudaFree(p->retry);
   cudaFree(p->table);
   cudaFree(p->item_start);

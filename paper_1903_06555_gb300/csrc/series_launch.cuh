@@ -6,9 +6,11 @@
 template <typename T, typename C>
 SeriesView<T> series_view(const Plan& p, int g) {
   SeriesView<T> v;
-  v.j0 = static_cast<const T*>(p.series_j0);
-  v.omn2 = p.series_omn2;
+  v.j0 = static_cast<const double*>(p.series_j0);
+  v.tiles_a = static_cast<const uint4*>(p.series_j0);
+  v.nodes = p.series_nodes;
   v.stride = p.series_stride;
+  v.tiles = p.series_stride / kSeriesTile;
   v.max_panels = p.series_max_panels;
   v.max_intervals = p.series_max_intervals;
   v.support = p.d.support;
@@ -45,24 +47,34 @@ int build_series_tables_t(Plan& p, cudaStream_t s) {
   }
   p.series_max_panels = std::min(panels, kSeriesMaxPanels);
   p.series_max_intervals = std::min(intervals, kSeriesMaxSamples - SeriesN<T>::half);
-  const int stride = (p.series_max_intervals + SeriesN<T>::half + 31) / 32 * 32;
+  const int grain = sizeof(T) == 4 ? kSeriesTile : 32;   // samples of a tile, of a warp
+  const int stride = (p.series_max_intervals + SeriesN<T>::half + grain - 1) / grain * grain;
   const int64_t rows = panel_table_offset(p.series_max_panels + 1);
+  const int panel_rows = series_panel_base(p.series_max_panels + 1);
+  const size_t table = sizeof(T) == 4 ? sizeof(uint4) * 128 * panel_rows * (stride / kSeriesTile)
+                                      : sizeof(double) * rows * stride;
   void* raw = nullptr;
-  PHI_CUDA_TRY(cudaMalloc(&raw, sizeof(T) * rows * stride));
+  PHI_CUDA_TRY(cudaMalloc(&raw, table));
   p.series_j0 = raw;
-  p.device_bytes += static_cast<int64_t>(sizeof(T) * rows * stride);
+  p.device_bytes += static_cast<int64_t>(table);
   if (sizeof(T) == 4) {
-    PHI_CUDA_TRY(cudaMalloc(&raw, sizeof(float2) * rows));
-    p.series_omn2 = static_cast<float2*>(raw);
-    p.device_bytes += static_cast<int64_t>(sizeof(float2) * rows);
+    const size_t bytes = sizeof(float4) * 32 * panel_rows;
+    PHI_CUDA_TRY(cudaMalloc(&raw, bytes));
+    p.series_nodes = static_cast<float4*>(raw);
+    p.device_bytes += static_cast<int64_t>(bytes);
   }
   PHI_CUDA_TRY(cudaMalloc(&raw, sizeof(uint32_t) * p.n_kept));
   p.retry = static_cast<uint32_t*>(raw);
   p.device_bytes += static_cast<int64_t>(sizeof(uint32_t) * p.n_kept);
-  const int blocks =
-      static_cast<int>(std::min<int64_t>((rows * stride + 255) / 256, p.num_sms * 8));
-  series_table_kernel<T><<<blocks, 256, 0, s>>>(p.node_omn, rows, stride,
-                                                static_cast<T*>(p.series_j0), p.series_omn2);
+  const int64_t items = sizeof(T) == 4 ? int64_t(panel_rows) * (stride / kSeriesTile) * 64
+                                       : rows * stride;
+  const int blocks = static_cast<int>(std::min<int64_t>((items + 127) / 128, p.num_sms * 16));
+  if (sizeof(T) == 4)
+    series_tile_kernel<<<blocks, 128, 0, s>>>(panel_rows, stride / kSeriesTile, p.node_omn,
+                                              static_cast<const float*>(p.node_hk),
+                                              static_cast<uint4*>(p.series_j0), p.series_nodes);
+  else
+    series_table_kernel<<<blocks, 128, 0, s>>>(rows, stride, static_cast<double*>(p.series_j0));
   PHI_CUDA_TRY(cudaGetLastError());
   p.series_stride = stride;
   return PHI_OK;
@@ -101,12 +113,17 @@ int series_shape(const Plan& p, K kernel, int64_t n, SeriesShape& sh) {
       per_sm < 1)
     per_sm = 1;
   sh.blocks = per_sm * p.num_sms;
-  // pairs are taken within a batch: batches of an even number once there are
-  // several visibilities to a warp, single visibilities before that
+  // FP32 samples the visibilities of a batch four at a time: batches of a
+  // multiple of four once there are several to a warp, smaller ones before
+  // that, so that every warp has work
   const int64_t warps = static_cast<int64_t>(sh.blocks) * sh.warps;
   sh.batch = queue_batch(n, warps);
-  if (sh.batch < 2 && n >= 4 * warps) sh.batch = 2;
-  if (sh.batch > 1) sh.batch &= ~1;
+  if (SeriesVis<T>::n > 1) {
+    if (sh.batch < 4)
+      sh.batch = static_cast<int>(std::min<int64_t>(4, std::max<int64_t>(1, n / (2 * warps))));
+    else
+      sh.batch = sh.batch / 4 * 4;
+  }
   return PHI_OK;
 }
 
