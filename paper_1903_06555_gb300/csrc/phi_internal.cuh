@@ -152,6 +152,7 @@ struct QuadParams {
   int max_refine;         // panel-count doublings allowed
   int npad;
   const double* node_omn;  // 1 - n(r_j) per node, all panel counts
+  const float2* node_omn2; // FP32: the same as the sum of two floats
   const void* node_hk;     // w_K(j) 2 pi h g(r_j) r_j per node (T)
   const void* node_hd;     // w_G(j) (FP32) or w_K(j) - w_G(j) (FP64), times 2 pi h g(r_j) r_j
   const uint16_t* tap_order;  // per even J_w: taps (a | b << 8) by distance from the box centre
@@ -176,6 +177,7 @@ struct Plan {
   double* omn_pix = nullptr;
   void* corr_pix = nullptr;
   double* node_omn = nullptr;
+  float2* node_omn2 = nullptr;          // FP32: behind node_omn, in its allocation
   void* node_hk = nullptr;
   void* node_hd = nullptr;
   uint16_t* tap_order = nullptr;
@@ -258,6 +260,7 @@ struct Plan {
     q.max_refine = d.max_refine;
     q.npad = npad;
     q.node_omn = node_omn;
+    q.node_omn2 = node_omn2;
     q.node_hk = node_hk;
     q.node_hd = node_hd;
     q.tap_order = tap_order;

@@ -243,7 +243,7 @@ __device__ double taper_g(double r, double a, double beta, double i0beta) {
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void node_table_kernel(double R, double du, double a, double beta, double* omn,
-                                  T* hk, T* hd, int64_t total) {
+                                  float2* omn2, T* hk, T* hd, int64_t total) {
   int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (j >= total) return;
   int npan = 1;
@@ -256,7 +256,12 @@ __global__ void node_table_kernel(double R, double du, double a, double beta, do
   double r = hw * (2.0 * p + 1.0 + gk_node(k));
   double l = r / du;
   double s = l * l;
-  omn[j] = s / (1.0 + sqrt(1.0 - s));
+  const double om = s / (1.0 + sqrt(1.0 - s));
+  omn[j] = om;
+  if (omn2) {
+    const float hi = static_cast<float>(om);
+    omn2[j] = make_float2(hi, static_cast<float>(om - static_cast<double>(hi)));
+  }
   double h = 2.0 * kPi * hw * taper_g(r, a, beta, cyl_bessel_i0(beta)) * r;
   hk[j] = static_cast<T>(gk_wk(k) * h);
   // FP32 quadrature forms its estimate from panel sums with the Gauss weight
@@ -283,11 +288,11 @@ int launch_node_tables(Plan& p, cudaStream_t s) {
   int blocks = static_cast<int>((total + 255) / 256);
   double a = 0.5 * p.d.support;
   if (p.d.precision == PHI_F64)
-    node_table_kernel<double><<<blocks, 256, 0, s>>>(p.R, p.du, a, p.beta, p.node_omn,
+    node_table_kernel<double><<<blocks, 256, 0, s>>>(p.R, p.du, a, p.beta, p.node_omn, nullptr,
                                                     static_cast<double*>(p.node_hk),
                                                     static_cast<double*>(p.node_hd), total);
   else
-    node_table_kernel<float><<<blocks, 256, 0, s>>>(p.R, p.du, a, p.beta, p.node_omn,
+    node_table_kernel<float><<<blocks, 256, 0, s>>>(p.R, p.du, a, p.beta, p.node_omn, p.node_omn2,
                                                    static_cast<float*>(p.node_hk),
                                                    static_cast<float*>(p.node_hd), total);
   PHI_CUDA_TRY(cudaGetLastError());
@@ -1459,32 +1464,127 @@ __global__ void __launch_bounds__(256) row_table_kernel(
   flush_counts(stats, 0, my_taps, 0, lane);
 }
 
-// phi_wkernel: one warp per point, lane 0 carries the tap.
-template <typename T, typename C>
-__global__ void __launch_bounds__(256) wkernel_kernel(const double* __restrict__ rho_in,
-                                                      const double* __restrict__ dw_in, int64_t n,
-                                                      C* __restrict__ out, QuadParams q,
-                                                      unsigned long long* bad) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  NodeVal<T>* sh = reinterpret_cast<NodeVal<T>*>(smem_raw) + warp * kNodeBatch;
-  const int64_t wpb = blockDim.x >> 5;
-  for (int64_t i = blockIdx.x * wpb + warp; i < n; i += (int64_t)gridDim.x * wpb) {
+// e^{2 pi i dw (1 - n)} in FP32: the phase from dw and 1 - n as sums of two
+// floats each (48 bits; the FP64 unit, at 1/64 of the FP32 rate, would take
+// longer than the quadrature it serves).
+struct PhaseF {
+  float hi, lo;
+  __device__ __forceinline__ explicit PhaseF(double dw) {
+    hi = static_cast<float>(dw);
+    lo = static_cast<float>(dw - static_cast<double>(hi));
+  }
+  __device__ __forceinline__ float2 operator()(float omn_hi, float omn_lo) const {
+    const float p = __fmul_rn(hi, omn_hi);
+    float e = fmaf(hi, omn_hi, -p);
+    e = fmaf(hi, omn_lo, e);
+    e = fmaf(lo, omn_hi, e);
+    float sn, cs;
+    sincospif(2.0f * ((p - rintf(p)) + e), &sn, &cs);
+    return make_float2(cs, sn);
+  }
+};
+
+// [GC] at arbitrary points (phi_wkernel and phi_wkernel_noalloc): every point
+// has its own |dw|, so nothing but the node table is shared.  L lanes take a
+// point, each the nodes k = sub, sub + L, ... of every panel, with the node
+// value and J0 formed together; per panel two shuffles over the L lanes make
+// the Kronrod-minus-Gauss sum for the estimate, refined as eval_chunk does
+// for a chunk of one tap.  (One warp per point, all lanes at the one tap,
+// repeated every Bessel function 32 times: 113 us for 40,009 points in FP32.)
+// Bound: FP32 issue, ~90 instructions per node.  L = 4 keeps the shuffles
+// below a tenth of that; 32 when there are too few points to fill the chip.
+template <typename T, typename C, int L>
+__device__ __forceinline__ void wkernel_points(const double* __restrict__ rho_in,
+                                               const double* __restrict__ dw_in, int64_t n,
+                                               C* __restrict__ out, const QuadParams& q,
+                                               int max_panels, unsigned long long* bad) {
+  const int lane = threadIdx.x & 31, sub = lane & (L - 1);
+  const unsigned group = (L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u)) << (lane & ~(L - 1));
+  const int64_t step = (int64_t)gridDim.x * blockDim.x / L;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / L; i < n; i += step) {
     const T rho = static_cast<T>(rho_in[i]);
     const double dw = dw_in[i];
-    int built = 0;
-    bool ok = true;
-    unsigned long long nodes = 0;
-    const C K = eval_chunk<T, C>(sh, q, rho, lane == 0, dw,
-                                 initial_panels(q, static_cast<float>(rho),
-                                                static_cast<float>(fabs(dw))),
-                                 kMaxPanels, built, ok, lane, nodes);
-    if (lane == 0) {
-      out[i] = K;
+    const PhaseF phase(dw);
+    int npan = min(initial_panels(q, static_cast<float>(rho), static_cast<float>(fabs(dw))),
+                   max_panels);
+    T kr, ki;
+    bool ok;
+    for (int refine = 0;; ++refine) {
+      const T Bh = sizeof(T) == 4 ? static_cast<T>(q.Rf / static_cast<float>(npan)) * rho
+                                  : static_cast<T>(panel_bh(q, rho, npan));
+      const int64_t off = panel_table_offset(npan);
+      T err = 0;
+      kr = ki = 0;
+      for (int p = 0; p < npan; ++p) {
+        const T a = Bh * static_cast<T>(2 * p + 1);
+        T dr = 0, di = 0;
+#pragma unroll 1
+        for (int k = sub; k < kNodes; k += L) {
+          const int64_t j = off + kNodes * p + k;
+          const T hk = static_cast<const T*>(q.node_hk)[j];
+          T hd = static_cast<const T*>(q.node_hd)[j];
+          C e;
+          if constexpr (sizeof(T) == 4) {
+            hd = hk - hd;   // FP32 tabulates the Gauss weight, FP64 the difference
+            const float2 om = q.node_omn2[j];
+            e = phase(om.x, om.y);
+          } else {
+            double t = dw * q.node_omn[j];
+            t -= rint(t);
+            sincos_pi(2.0 * t, &e.y, &e.x);
+          }
+          const T J = j0_hc(fma(Bh, gk_node_c(T(0), k), a));
+          kr = fma(J * hk, e.x, kr);
+          ki = fma(J * hk, e.y, ki);
+          dr = fma(J * hd, e.x, dr);
+          di = fma(J * hd, e.y, di);
+        }
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) {
+          dr += __shfl_xor_sync(group, dr, o);
+          di += __shfl_xor_sync(group, di, o);
+        }
+        err += est_sqrt(dr * dr + di * di);
+      }
+#pragma unroll
+      for (int o = L / 2; o > 0; o >>= 1) {
+        kr += __shfl_xor_sync(group, kr, o);
+        ki += __shfl_xor_sync(group, ki, o);
+      }
+      ok = err <= fmax(static_cast<T>(q.tol_abs),
+                       static_cast<T>(q.tol_rel) * est_sqrt(kr * kr + ki * ki));
+      if (ok || refine >= q.max_refine || npan >= max_panels) break;
+      npan = min(2 * npan, max_panels);
+    }
+    if (sub == 0) {
+      out[i] = cmake<C>(kr, ki);
       if (!ok) atomicAdd(bad, 1ULL);
     }
   }
+}
+
+template <typename T, typename C, int L>
+__global__ void __launch_bounds__(256) wkernel_kernel(const double* __restrict__ rho_in,
+                                                      const double* __restrict__ dw_in, int64_t n,
+                                                      C* __restrict__ out, QuadParams q,
+                                                      int max_panels, unsigned long long* bad) {
+  wkernel_points<T, C, L>(rho_in, dw_in, n, out, q, max_panels, bad);
+}
+
+// Four lanes per point once that gives every SM two warps or more, a warp
+// per point below.
+template <typename T, typename C>
+cudaError_t launch_wkernel(const double* rho, const double* dw, int64_t n, C* out,
+                           const QuadParams& q, int max_panels, unsigned long long* bad,
+                           int num_sms, cudaStream_t s) {
+  const bool wide = n < 16 * (int64_t)num_sms;
+  const int64_t want = (n * (wide ? 32 : 4) + 255) / 256;
+  const int blocks = static_cast<int>(std::min<int64_t>(want, 65535));
+  if (wide)
+    wkernel_kernel<T, C, 32><<<blocks, 256, 0, s>>>(rho, dw, n, out, q, max_panels, bad);
+  else
+    wkernel_kernel<T, C, 4><<<blocks, 256, 0, s>>>(rho, dw, n, out, q, max_panels, bad);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -2095,11 +2195,7 @@ int run_wkernel(Plan& p, const double* rho, const double* dw, int64_t n, C* out,
   unsigned long long* bad = p.counters + p.K + 2;
   PHI_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(unsigned long long), s));
   if (n > 0) {
-    const size_t smem = (kVisThreads / 32) * kNodeBatch * sizeof(NodeVal<T>);
-    int64_t want = (n + 7) / 8;
-    int blocks = static_cast<int>(want < 65535 ? want : 65535);
-    wkernel_kernel<T, C><<<blocks, kVisThreads, smem, s>>>(rho, dw, n, out, p.quad(), bad);
-    PHI_CUDA_TRY(cudaGetLastError());
+    PHI_CUDA_TRY((launch_wkernel<T, C>(rho, dw, n, out, p.quad(), kMaxPanels, bad, p.num_sms, s)));
   }
   if (n_bad) {
     unsigned long long h = 0;
@@ -2208,13 +2304,9 @@ int set_kernel_smem_limits() {
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f32));
   PHI_CUDA_TRY(cudaFuncSetAttribute(vis_kernel<float, float2, true>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f32));
-  PHI_CUDA_TRY(cudaFuncSetAttribute(wkernel_kernel<float, float2>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f32));
   PHI_CUDA_TRY(cudaFuncSetAttribute(vis_kernel<double, double2, false>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f64));
   PHI_CUDA_TRY(cudaFuncSetAttribute(vis_kernel<double, double2, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f64));
-  PHI_CUDA_TRY(cudaFuncSetAttribute(wkernel_kernel<double, double2>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f64));
   PHI_CUDA_TRY(cudaFuncSetAttribute(table_sample_kernel<float, float2>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f32));
@@ -2402,46 +2494,21 @@ int noalloc_scratch(unsigned char** out) {
 }
 
 template <typename T, typename C>
-__global__ void __launch_bounds__(256) wkernel_noalloc_kernel(const double* __restrict__ rho_in,
-                                                              const double* __restrict__ dw_in,
-                                                              int64_t n, C* __restrict__ out,
-                                                              QuadParams q, int max_panels,
-                                                              unsigned long long* bad) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  NodeVal<T>* sh = reinterpret_cast<NodeVal<T>*>(smem_raw) + warp * kNodeBatch;
-  const int64_t wpb = blockDim.x >> 5;
-  for (int64_t i = blockIdx.x * wpb + warp; i < n; i += (int64_t)gridDim.x * wpb) {
-    const T rho = static_cast<T>(rho_in[i]);
-    const double dw = dw_in[i];
-    int built = 0;
-    bool ok = true;
-    unsigned long long nodes = 0;
-    const C K = eval_chunk<T, C>(
-        sh, q, rho, lane == 0, dw,
-        initial_panels(q, static_cast<float>(rho), static_cast<float>(fabs(dw))), max_panels,
-        built, ok, lane, nodes);
-    if (lane == 0) {
-      out[i] = K;
-      if (!ok) atomicAdd(bad, 1ULL);
-    }
-  }
-}
-
-template <typename T, typename C>
 int run_wkernel_noalloc(const phi_wkernel_params& prm, const double* rho, const double* dw,
                         int64_t n, C* out, int64_t* n_bad, cudaStream_t s) {
   unsigned char* base = nullptr;
   int st = noalloc_scratch(&base);
   if (st != PHI_OK) return st;
-  const size_t smem = (kVisThreads / 32) * kNodeBatch * sizeof(NodeVal<T>);
-  PHI_CUDA_TRY(cudaFuncSetAttribute(wkernel_noalloc_kernel<T, C>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int dev = 0, num_sms = 0;
+  PHI_CUDA_TRY(cudaGetDevice(&dev));
+  PHI_CUDA_TRY(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
   unsigned long long* bad = reinterpret_cast<unsigned long long*>(base);
   double* omn = reinterpret_cast<double*>(base + 256);
+  // FP32: both weights in the second third, 1 - n in two floats in the last
+  const bool f32 = sizeof(T) == 4;
   T* hk = reinterpret_cast<T*>(base + 256 + 8 * kNoAllocNodes);
-  T* hd = reinterpret_cast<T*>(base + 256 + 16 * kNoAllocNodes);
+  T* hd = f32 ? hk + kNoAllocNodes : reinterpret_cast<T*>(base + 256 + 16 * kNoAllocNodes);
+  float2* omn2 = f32 ? reinterpret_cast<float2*>(base + 256 + 16 * kNoAllocNodes) : nullptr;
   const int64_t nodes = panel_table_offset(prm.max_panels + 1);
   const double l_win = prm.window_radius / prm.du;
   const double n_win = sqrt(1.0 - l_win * l_win);
@@ -2455,6 +2522,7 @@ int run_wkernel_noalloc(const phi_wkernel_params& prm, const double* rho, const 
   q.max_refine = prm.max_refine;
   q.npad = 0;
   q.node_omn = omn;
+  q.node_omn2 = omn2;
   q.node_hk = hk;
   q.node_hd = hd;
   q.tap_order = nullptr;
@@ -2462,14 +2530,10 @@ int run_wkernel_noalloc(const phi_wkernel_params& prm, const double* rho, const 
   // the counter keeps the previous call's value: clear it first
   PHI_CUDA_TRY(cudaMemsetAsync(bad, 0, sizeof(unsigned long long), s));
   node_table_kernel<T><<<static_cast<int>((nodes + 255) / 256), 256, 0, s>>>(
-      prm.window_radius, prm.du, 0.5 * prm.support, prm.kb_beta, omn, hk, hd, nodes);
+      prm.window_radius, prm.du, 0.5 * prm.support, prm.kb_beta, omn, omn2, hk, hd, nodes);
   PHI_CUDA_TRY(cudaGetLastError());
   if (n > 0) {
-    const int64_t want = (n + 7) / 8;
-    const int blocks = static_cast<int>(want < 65535 ? want : 65535);
-    wkernel_noalloc_kernel<T, C><<<blocks, kVisThreads, smem, s>>>(rho, dw, n, out, q,
-                                                                   prm.max_panels, bad);
-    PHI_CUDA_TRY(cudaGetLastError());
+    PHI_CUDA_TRY((launch_wkernel<T, C>(rho, dw, n, out, q, prm.max_panels, bad, num_sms, s)));
   }
   if (n_bad) {
     unsigned long long h = 0;

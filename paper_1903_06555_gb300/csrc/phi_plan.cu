@@ -775,7 +775,8 @@ int build(Plan& p, const double* uvw, const double* weights, int64_t M, cudaStre
   // --- tables, grid, FFT plan
   const size_t tsize = f64 ? sizeof(double) : sizeof(float);
   const int64_t nodes = panel_table_offset(kMaxPanels + 1);
-  PHI_CUDA_TRY(owned_alloc(p, &p.node_omn, nodes));
+  PHI_CUDA_TRY(owned_alloc(p, &p.node_omn, f64 ? nodes : 2 * nodes));
+  if (!f64) p.node_omn2 = reinterpret_cast<float2*>(p.node_omn + nodes);
   PHI_CUDA_TRY(owned_alloc(p, reinterpret_cast<unsigned char**>(&p.node_hk), tsize * nodes));
   PHI_CUDA_TRY(owned_alloc(p, reinterpret_cast<unsigned char**>(&p.node_hd), tsize * nodes));
   PHI_TRY(build_tap_order(p, std::max(p.max_jw, 2), s));

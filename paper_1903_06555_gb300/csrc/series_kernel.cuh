@@ -35,6 +35,12 @@
 // table loads and two broadcasts per node and pair of visibilities).  FP64
 // walks the nodes, one sample per lane.
 //
+// FP32 makes the sums on the tensor cores (series_tile_kernel says how the
+// operands are split), four visibilities of one panel count to a warp: 1.3 ms
+// of the snapshot's launch where one FP32 product per lane took 3.9 (two
+// table loads and two broadcasts per node and pair of visibilities).  FP64
+// walks the nodes, one sample per lane.
+//
 // Measured on the MWA-like snapshot (1.92M visibilities, J_w 26-40, FP32):
 // 5.4 ms per degrid or grid launch where the per-tap kernel takes 63 and the
 // 16-point radial series 18.6, and 4.2e-7 from the 64-bit operator (per tap
@@ -163,25 +169,6 @@ __global__ void series_tile_kernel(int panels, int tiles, const double* __restri
     }
   }
 }
-
-// e^{2 pi i dw (1 - n)} in FP32: the phase from dw and 1 - n as sums of two
-// floats each (48 bits; the FP64 unit would take as long as the sampling).
-struct PhaseF {
-  float hi, lo;
-  __device__ __forceinline__ explicit PhaseF(double dw) {
-    hi = static_cast<float>(dw);
-    lo = static_cast<float>(dw - static_cast<double>(hi));
-  }
-  __device__ __forceinline__ float2 operator()(float omn_hi, float omn_lo) const {
-    const float p = __fmul_rn(hi, omn_hi);
-    float e = fmaf(hi, omn_hi, -p);
-    e = fmaf(hi, omn_lo, e);
-    e = fmaf(lo, omn_hi, e);
-    float sn, cs;
-    sincospif(2.0f * ((p - rintf(p)) + e), &sn, &cs);
-    return make_float2(cs, sn);
-  }
-};
 
 __device__ __forceinline__ void series_mma(float (&c)[4], const uint4& a, const unsigned (&b)[2]) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
