@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) vis_dde_kernel(
     const C* __restrict__ grid_in, C* grid_out, const C* __restrict__ vis_in,
     C* __restrict__ vis_out, QuadParams q, RadialView<T> rv, const C* __restrict__ dde_a,
     const C* __restrict__ dde_b, int jd, int jmax, const int32_t* __restrict__ stack_slot,
-    unsigned long long* head, unsigned long long* stats, int batch) {
+    unsigned long long* head, unsigned long long* stats, int batch, RecordList list) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -80,9 +80,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) vis_dde_kernel(
                 "the per-lane ring of the largest DDE kernel must fit the node buffer");
   unsigned long long my_bad = 0, my_taps = 0, my_nodes = 0;
   const int npad = q.npad;
+  n = list.count(n);
   WarpQueue wq;
   unsigned long long i;
   while (wq.take(head, static_cast<unsigned long long>(batch), n, lane, i)) {
+    i = list.record(i);
     const VisRec<T> r = recs[i];
     const int Jw = r.jw, Jc = Jw + 2 * h;
     const int64_t gbase = static_cast<int64_t>(stack_slot[r.stack]) * npad * npad;
@@ -225,17 +227,15 @@ template <typename T, typename C>
 __global__ void __launch_bounds__(VisLaunch<T>::threads, VisLaunch<T>::min_blocks)
     dde_box_kernel(const VisRec<T>* __restrict__ recs, int64_t n, C* __restrict__ boxes,
                    int jmax, QuadParams q, unsigned long long* head,
-                   unsigned long long* stats, int batch, RecordList list) {
+                   unsigned long long* stats, int batch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   NodeVal<T>* sh = reinterpret_cast<NodeVal<T>*>(smem_raw) + warp * kNodeBatch;
   unsigned long long my_bad = 0, my_nodes = 0;
-  n = list.count(n);
   WarpQueue wq;
   unsigned long long i;
   while (wq.take(head, static_cast<unsigned long long>(batch), n, lane, i)) {
-    i = list.record(i);
     const VisRec<T> r = recs[i];
     const int Jw = r.jw, half = Jw / 2, ntap = Jw * Jw;
     C* box = boxes + static_cast<int64_t>(i) * jmax * jmax;
@@ -291,8 +291,7 @@ __global__ void __launch_bounds__(VisLaunch<T>::threads, VisLaunch<T>::min_block
 template <typename T, typename C>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) dde_box_radial_kernel(
     const VisRec<T>* __restrict__ recs, int64_t n, C* __restrict__ boxes, int jmax, QuadParams q,
-    RadialView<T> rv, unsigned long long* head, unsigned long long* stats, int batch,
-    RecordList list) {
+    RadialView<T> rv, unsigned long long* head, unsigned long long* stats, int batch) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -300,11 +299,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) dde_box_radial_ke
   C* ser = reinterpret_cast<C*>(smem_raw + (blockDim.x >> 5) * kNodeBatch * sizeof(NodeVal<T>)) +
            warp * rv.buf;
   unsigned long long my_bad = 0, my_nodes = 0;
-  n = list.count(n);
   WarpQueue wq;
   unsigned long long i;
   while (wq.take(head, static_cast<unsigned long long>(batch), n, lane, i)) {
-    i = list.record(i);
     const VisRec<T> r = recs[i];
     const int Jw = r.jw, half = Jw / 2, ntap = Jw * Jw;
     C* box = boxes + static_cast<int64_t>(i) * jmax * jmax;
@@ -417,4 +414,162 @@ __global__ void __launch_bounds__(256) dde_conv_kernel(
     if (!kGrid) store_visibility<T, C>(accv, static_cast<T>(r.weight), pm, vis_out, lane);
   }
   flush_counts(stats, 0, my_taps, 0, lane);
+}
+
+// The DDE convolution of the sampled quadrature (series_kernel.cuh): the taps
+// come cheaply from the visibility's polynomials, so the warp walks the box
+// in bands of four rows, kept in shared memory with the ring of row-pass rows
+// the column pass still needs: (a) the band's taps into `band`, 2 h zeros
+// either side of each row; (b) R(kb, cu) = sum_s a_s K(kb, cu - 2 h + s) of
+// its rows into ring row kb mod (4 + 2 h); (c) the combined rows cv = k0 ..
+// k0 + 3, C(cv, cu) = sum_s b_s R(cv - 2 h + s, cu), applied to the grid.
+// Rows outside the box are zeros in the ring.
+constexpr int kDdeRows = 4;
+__host__ __device__ inline int dde_series_elems(int jmax, int jd) {
+  const int h2 = jd - 1;
+  return 2 * jd + kDdeRows * (jmax + 2 * h2) + (kDdeRows + h2) * (jmax + h2);
+}
+// acc + i acc2 accumulates a k as a.x k and a.y k apart.
+__device__ __forceinline__ void cmad_parts(float2& acc, float2& acc2, const float2& a,
+                                           const float2& k) {
+  acc = __ffma2_rn(make_float2(a.x, a.x), k, acc);
+  acc2 = __ffma2_rn(make_float2(a.y, a.y), k, acc2);
+}
+__device__ __forceinline__ void cmad_parts(double2& acc, double2& acc2, const double2& a,
+                                           const double2& k) {
+  acc.x = fma(a.x, k.x, acc.x);
+  acc.y = fma(a.x, k.y, acc.y);
+  acc2.x = fma(a.y, k.x, acc2.x);
+  acc2.y = fma(a.y, k.y, acc2.y);
+}
+template <typename T, typename C, bool kGrid>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) dde_series_kernel(
+    const VisRec<T>* __restrict__ recs, const uint32_t* __restrict__ perm, int64_t n,
+    const C* __restrict__ grid_in, C* grid_out, const C* __restrict__ vis_in,
+    C* __restrict__ vis_out, QuadParams q, SeriesView<T> sv, const C* __restrict__ dde_a,
+    const C* __restrict__ dde_b, int jd, int jmax, const int32_t* __restrict__ stack_slot,
+    unsigned long long* head, unsigned long long* stats, int batch) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31;
+  const int series_bytes = series_warp_bytes<T>(sv.stride, sv.max_intervals);
+  unsigned char* base = smem_raw + (threadIdx.x >> 5) *
+                        (series_bytes + dde_series_elems(jmax, jd) * static_cast<int>(sizeof(C)));
+  SeriesWarp<T, C> w(base, sv);
+  const int h = jd >> 1, h2 = 2 * h, nring = kDdeRows + h2;
+  const int bw = jmax + 2 * h2, rw = jmax + h2;   // row lengths of the band and the ring
+  C* dab = reinterpret_cast<C*>(base + series_bytes);   // a_i then b_i
+  C* band = dab + 2 * jd;
+  C* ring = band + kDdeRows * bw;
+  unsigned long long my_taps = 0, my_nodes = 0;
+  const int npad = q.npad;
+  const C zero = cmake<C>(0.0, 0.0);
+  WarpQueue wq;
+  unsigned long long i0;
+  int nv, pass, P;
+  while (series_take<T, C>(w, wq, head, static_cast<unsigned long long>(batch), n, recs, sv, q,
+                           lane, i0, nv, pass, P)) {
+#pragma unroll 1
+    for (int v = 0; v < nv; ++v) {
+      if (!((pass >> v) & 1)) continue;
+      const VisRec<T> r = recs[i0 + v];
+      const int Jw = r.jw, Jc = Jw + h2, half = Jw / 2;
+      const int NP = series_intervals(r.jw, sv.inv_delta_f);
+      w.polynomials(v, NP, lane);
+      const int64_t gbase = static_cast<int64_t>(stack_slot[r.stack]) * npad * npad;
+      const uint32_t pm = perm[i0 + v];
+      const int64_t src = pm & 0x7fffffffu;
+      const C yv = kGrid ? load_visibility<T, C>(vis_in, pm, static_cast<T>(r.weight)) : zero;
+      if (lane < 2 * jd)
+        dab[lane] = lane < jd ? dde_a[src * jd + lane] : dde_b[src * jd + lane - jd];
+      for (int e = lane; e < kDdeRows * h2; e += 32) {   // the band's zeros, 2 h to a side
+        const int row = e / h2, s = e - row * h2;
+        band[row * bw + s] = zero;
+        band[row * bw + h2 + Jw + s] = zero;
+      }
+      for (int e = lane; e < nring * rw; e += 32) ring[e] = zero;
+      C accv = zero;
+      // box origin on the grid; columns and rows wrap by one conditional
+      const int u0 = r.bu - h - half + 1, v0 = r.bv - h - half + 1;
+      const int step_r = 32 / Jc, step_c = 32 % Jc;
+      int slot0 = nring - h2;                            // ring row of kb = k0 - 2 h
+      for (int k0 = 0; k0 < Jc; k0 += kDdeRows) {
+        __syncwarp();
+        // (a) the taps of rows k0 .. k0 + 3; rows past the box are zeros
+        if constexpr (sizeof(T) == 4) {
+          const int row = 2 * ((lane >> 3) & 1);
+          const float nb = static_cast<float>(half - 1 - k0 - row);
+          const float2 dv_ = __fadd2_rn(make_float2(r.fv, r.fv), make_float2(nb, nb - 1.0f));
+          for (int a = (lane & 7) | ((lane & 16) >> 1); a < Jw; a += 16) {
+            const float du_ = r.fu + static_cast<float>(half - 1 - a), d2 = du_ * du_;
+            float2 t0 = zero, t1 = zero;
+            if (k0 + row < Jw)
+              series_eval2(w.coef, w.slots, sv.inv_delta,
+                           __ffma2_rn(dv_, dv_, make_float2(d2, d2)), t0, t1);
+            band[row * bw + h2 + a] = t0;
+            band[(row + 1) * bw + h2 + a] = t1;
+          }
+        } else {
+          for (int e = lane; e < kDdeRows * Jw; e += 32) {
+            const int row = e / Jw, a = e - row * Jw;
+            const T du_ = r.fu - static_cast<T>(a - half + 1);
+            const T dv_ = r.fv - static_cast<T>(k0 + row - half + 1);
+            C t = zero;
+            if (k0 + row < Jw) t = series_eval(w.coef, w.slots, sv.inv_delta, du_ * du_ + dv_ * dv_);
+            band[row * bw + h2 + a] = t;
+          }
+        }
+        __syncwarp();
+        // (b) their rows of R; slot1: the ring row of kb = k0
+        int slot1 = slot0 + h2;
+        if (slot1 >= nring) slot1 -= nring;
+        for (int rr = lane / Jc, cu = lane - rr * Jc; rr < kDdeRows;) {
+          const C* k = band + rr * bw + cu;
+          C acc = zero, acc2 = zero;
+#pragma unroll 5
+          for (int s = 0; s < jd; ++s) cmad_parts(acc, acc2, dab[s], k[s]);
+          int sl = slot1 + rr;
+          if (sl >= nring) sl -= nring;
+          acc.x -= acc2.y;
+          acc.y += acc2.x;
+          ring[sl * rw + cu] = acc;
+          rr += step_r;
+          cu += step_c;
+          if (cu >= Jc) {
+            cu -= Jc;
+            ++rr;
+          }
+        }
+        __syncwarp();
+        // (c) the combined rows k0 .. k0 + 3
+        for (int rr = lane / Jc, cu = lane - rr * Jc; rr < kDdeRows && k0 + rr < Jc;) {
+          C acc = zero, acc2 = zero;
+          int sl = slot0 + rr;
+          if (sl >= nring) sl -= nring;
+#pragma unroll 5
+          for (int s = 0; s < jd; ++s) {
+            cmad_parts(acc, acc2, dab[jd + s], ring[sl * rw + cu]);
+            sl = sl + 1 == nring ? 0 : sl + 1;
+          }
+          acc.x -= acc2.y;
+          acc.y += acc2.x;
+          ++my_taps;
+          apply_tap<C, kGrid>(acc, gbase + static_cast<int64_t>(wrap_index(v0 + k0 + rr, npad)) * npad +
+                                       wrap_index(u0 + cu, npad),
+                              yv, grid_in, grid_out, q.fx, accv);
+          rr += step_r;
+          cu += step_c;
+          if (cu >= Jc) {
+            cu -= Jc;
+            ++rr;
+          }
+        }
+        slot0 += kDdeRows;
+        if (slot0 >= nring) slot0 -= nring;
+      }
+      if (lane == 0) my_nodes += static_cast<unsigned long long>((NP + 1) * kNodes * P);
+      if (!kGrid) store_visibility<T, C>(accv, static_cast<T>(r.weight), pm, vis_out, lane);
+      __syncwarp();   // the polynomials, the band and the ring are rewritten
+    }
+  }
+  flush_counts(stats, 0, my_taps, my_nodes, lane);
 }

@@ -46,7 +46,6 @@ int launch_dde_two_pass(Plan& p, const VisRec<T>* recs, int64_t b0, int64_t nk, 
   // pass 1: the plain kernel's block shape and shared memory (limits set
   // to one value for all plans, so concurrent launchers agree)
   const bool radial = p.d.kernel_mode == PHI_KERNEL_RADIAL;
-  const bool series = p.series_stride > 0;
   constexpr int box_threads = VisLaunch<T>::threads;
   const size_t box_smem = radial ? radial_smem<T, C>(p)
                                  : (box_threads / 32) * kNodeBatch * sizeof(NodeVal<T>);
@@ -86,28 +85,14 @@ int launch_dde_two_pass(Plan& p, const VisRec<T>* recs, int64_t b0, int64_t nk, 
       st = PHI_ERR_CUDA;
       break;
     }
-    // the boxes at the samples in rho, then the records those left
-    RecordList list{nullptr, nullptr};
-    unsigned long long* box_head = head;
-    int batch = queue_batch(n, box_blocks * (box_threads / 32));
-    if (series) {
-      box_head = p.retry_counters + 2 * g + 1;
-      if (cudaMemsetAsync(p.retry_counters + 2 * g, 0, 2 * sizeof(unsigned long long), s) !=
-              cudaSuccess ||
-          launch_box_series<T, C>(p, g, recs + c0, n, boxes, jmax, s) != PHI_OK) {
-        st = PHI_ERR_CUDA;
-        break;
-      }
-      list = RecordList{p.retry, p.retry_counters + 2 * g};
-      batch = 1;
-    }
     if (radial)
       dde_box_radial_kernel<T, C><<<box_blocks, box_threads, box_smem, s>>>(
-          recs + c0, n, boxes, jmax, p.quad(), radial_view<T, C>(p), box_head, p.counters + p.K,
-          batch, list);
+          recs + c0, n, boxes, jmax, p.quad(), radial_view<T, C>(p), head, p.counters + p.K,
+          queue_batch(n, box_blocks * (box_threads / 32)));
     else
       dde_box_kernel<T, C><<<box_blocks, box_threads, box_smem, s>>>(
-          recs + c0, n, boxes, jmax, p.quad(), box_head, p.counters + p.K, batch, list);
+          recs + c0, n, boxes, jmax, p.quad(), head, p.counters + p.K,
+          queue_batch(n, box_blocks * (box_threads / 32)));
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemsetAsync(head, 0, sizeof(unsigned long long), s) != cudaSuccess) {
       st = PHI_ERR_CUDA;
@@ -122,6 +107,26 @@ int launch_dde_two_pass(Plan& p, const VisRec<T>* recs, int64_t b0, int64_t nk, 
   const cudaError_t ef = cudaFreeAsync(boxes, s);
   if (st != PHI_OK) return st;
   PHI_CUDA_TRY(ef);
+  return PHI_OK;
+}
+
+// The fused kernel of the sampled quadrature; `launched` false (and nothing
+// launched) when one warp's storage does not fit a block.
+template <typename T, typename C, bool kGrid>
+int launch_dde_series(Plan& p, int g, const VisRec<T>* recs, int64_t b0, int64_t nk,
+                      const C* grids_in, C* grids_out, const C* vis_in, C* vis_out,
+                      const DdeArgs& dde, cudaStream_t s, bool& launched) {
+  const int jmax = std::max(p.max_jw, 2);
+  const size_t extra = sizeof(C) * static_cast<size_t>(dde_series_elems(jmax, dde.jd));
+  SeriesShape sh;
+  PHI_TRY_ST((series_shape<T, C>(p, dde_series_kernel<T, C, kGrid>, nk, extra, sh)));
+  launched = sh.warps > 0;
+  if (!launched) return PHI_OK;
+  dde_series_kernel<T, C, kGrid><<<sh.blocks, 32 * sh.warps, sh.smem, s>>>(
+      recs, p.perm + b0, nk, grids_in, grids_out, vis_in, vis_out, p.quad(),
+      series_view<T, C>(p, g), static_cast<const C*>(dde.a), static_cast<const C*>(dde.b), dde.jd,
+      jmax, p.stack_slot_dev, p.counters + g, p.counters + p.K, sh.batch);
+  PHI_CUDA_TRY(cudaGetLastError());
   return PHI_OK;
 }
 
@@ -148,7 +153,21 @@ int launch_dde(Plan& p, const VisRec<T>* recs, int64_t b0, int64_t nk, int g, co
     }
   }
   const bool radial = p.d.kernel_mode == PHI_KERNEL_RADIAL;
-  if (best < kDdeTwoPassWarps) {
+  // the sampled quadrature where the plan has its tables, the single-pass
+  // kernel taking the visibilities it leaves (so only while their box fits a
+  // block); no buffer, and faster than either path below at every support
+  RecordList list{nullptr, nullptr};
+  unsigned long long* head = p.counters + g;
+  bool series = false;
+  if (p.series_stride > 0 && warps >= 1) {
+    PHI_TRY_ST((launch_dde_series<T, C, kGrid>(p, g, recs, b0, nk, grids_in, grids_out, vis_in,
+                                               vis_out, dde, s, series)));
+    if (series) {
+      list = RecordList{p.retry, p.retry_counters + 2 * g};
+      head = p.retry_counters + 2 * g + 1;
+    }
+  }
+  if (!series && best < kDdeTwoPassWarps) {
     bool launched = false;
     PHI_TRY_ST((launch_dde_two_pass<T, C, kGrid>(p, recs, b0, nk, g, grids_in, grids_out, vis_in,
                                                  vis_out, dde, s, launched)));
@@ -167,7 +186,7 @@ int launch_dde(Plan& p, const VisRec<T>* recs, int64_t b0, int64_t nk, int g, co
   kernel<<<blocks, 32 * warps, smem, s>>>(
       recs, p.perm + b0, nk, grids_in, grids_out, vis_in, vis_out, p.quad(), rv,
       static_cast<const C*>(dde.a), static_cast<const C*>(dde.b), dde.jd, std::max(p.max_jw, 2),
-      p.stack_slot_dev, p.counters + g, p.counters + p.K, queue_batch(nk, blocks * warps));
+      p.stack_slot_dev, head, p.counters + p.K, series ? 1 : queue_batch(nk, blocks * warps), list);
   PHI_CUDA_TRY(cudaGetLastError());
   return PHI_OK;
 }

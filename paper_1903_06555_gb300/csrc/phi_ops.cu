@@ -1787,7 +1787,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) vis_radial_kernel
   flush_counts(stats, my_bad, my_taps, my_nodes, lane);
 }
 
-// The quadrature at samples in rho: vis_series_kernel, dde_box_series_kernel
+// The quadrature at samples in rho: vis_series_kernel
 #include "series_kernel.cuh"
 
 // Direction-dependent effects (Sec. 5.2): vis_dde_kernel
@@ -2263,7 +2263,8 @@ cudaError_t set_series_smem(int bytes) {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaFuncSetAttribute(vis_series_kernel<T, C, false>, a, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(vis_series_kernel<T, C, true>, a, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(dde_box_series_kernel<T, C>, a, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(dde_series_kernel<T, C, false>, a, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(dde_series_kernel<T, C, true>, a, bytes);
   return e;
 }
 

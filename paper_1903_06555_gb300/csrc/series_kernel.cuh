@@ -737,50 +737,3 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
   }
   flush_counts(stats, 0, my_taps, my_nodes, lane);
 }
-
-// The J_w x J_w kernel box of each of records [0, n) into boxes[i * jmax^2],
-// row-major with row length J_w (pass 1 of the two-pass DDE convolution).
-template <typename T, typename C>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
-    dde_box_series_kernel(const VisRec<T>* __restrict__ recs, int64_t n, C* __restrict__ boxes,
-                          int jmax, QuadParams q, SeriesView<T> sv, unsigned long long* head,
-                          unsigned long long* stats, int batch) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int lane = threadIdx.x & 31;
-  SeriesWarp<T, C> w(smem_raw + (threadIdx.x >> 5) *
-                                    series_warp_bytes<T>(sv.stride, sv.max_intervals), sv);
-  unsigned long long my_nodes = 0;
-  WarpQueue wq;
-  unsigned long long i0;
-  int nv, pass, P;
-  while (series_take<T, C>(w, wq, head, static_cast<unsigned long long>(batch), n, recs, sv, q,
-                           lane, i0, nv, pass, P)) {
-#pragma unroll 1
-    for (int v = 0; v < nv; ++v) {
-      if (!((pass >> v) & 1)) continue;
-      const VisRec<T> rv = recs[i0 + v];
-      const int NP = series_intervals(rv.jw, sv.inv_delta_f);
-      w.polynomials(v, NP, lane);
-      const int Jw = rv.jw, half = Jw / 2, ntap = Jw * Jw;
-      C* box = boxes + static_cast<int64_t>(i0 + v) * jmax * jmax;
-      int a = lane % Jw, b = lane / Jw;
-      const int step_b = 32 / Jw, step_a = 32 % Jw;
-      for (int t = lane; t < ntap; t += 32) {
-        const T du_ = rv.fu - static_cast<T>(a - half + 1);
-        const T dv_ = rv.fv - static_cast<T>(b - half + 1);
-        box[t] = series_eval(w.coef, w.slots, sv.inv_delta, du_ * du_ + dv_ * dv_);
-        a += step_a;
-        b += step_b;
-        if (a >= Jw) {
-          a -= Jw;
-          ++b;
-        }
-      }
-      if (lane == 0) my_nodes += static_cast<unsigned long long>((NP + 1) * kNodes * P);
-      __syncwarp();
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) my_nodes += __shfl_xor_sync(0xffffffffu, my_nodes, o);
-  if (lane == 0 && my_nodes) atomicAdd(stats + 3, my_nodes);
-}

@@ -81,14 +81,15 @@ int build_series_tables_t(Plan& p, cudaStream_t s) {
 }
 
 // Block shape: as many warps per block (at most 8) as keep the most warps
-// resident, each with its own samples and polynomials.
+// resident, each with its own samples and polynomials and `extra` bytes; no
+// warps when one does not fit.
 struct SeriesShape {
   int warps = 0, blocks = 0, batch = 1;
   size_t smem = 0;
 };
 template <typename T, typename C, typename K>
-int series_shape(const Plan& p, K kernel, int64_t n, SeriesShape& sh) {
-  const size_t per_warp = series_warp_bytes<T>(p.series_stride, p.series_max_intervals);
+int series_shape(const Plan& p, K kernel, int64_t n, size_t extra, SeriesShape& sh) {
+  const size_t per_warp = series_warp_bytes<T>(p.series_stride, p.series_max_intervals) + extra;
   int dev = 0, optin = 0, per_sm_smem = 0, reserved = 0;
   PHI_CUDA_TRY(cudaGetDevice(&dev));
   PHI_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
@@ -105,7 +106,7 @@ int series_shape(const Plan& p, K kernel, int64_t n, SeriesShape& sh) {
       sh.warps = w;
     }
   }
-  if (sh.warps == 0) return PHI_ERR_SUPPORT;   // not reached: one warp takes 31 KB at most
+  if (sh.warps == 0) return PHI_OK;
   sh.smem = per_warp * sh.warps;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * sh.warps, sh.smem) !=
@@ -132,23 +133,11 @@ template <typename T, typename C, bool kGrid>
 int launch_series(Plan& p, int g, const VisRec<T>* recs, int64_t b0, int64_t nk, const C* grids_in,
                   C* grids_out, const C* vis_in, C* vis_out, cudaStream_t s) {
   SeriesShape sh;
-  PHI_TRY_ST((series_shape<T, C>(p, vis_series_kernel<T, C, kGrid>, nk, sh)));
+  PHI_TRY_ST((series_shape<T, C>(p, vis_series_kernel<T, C, kGrid>, nk, 0, sh)));
+  if (sh.warps == 0) return PHI_ERR_SUPPORT;   // not reached: one warp takes 31 KB at most
   vis_series_kernel<T, C, kGrid><<<sh.blocks, 32 * sh.warps, sh.smem, s>>>(
       recs, p.perm + b0, nk, grids_in, grids_out, vis_in, vis_out, p.quad(),
       series_view<T, C>(p, g), p.stack_slot_dev, p.counters + g, p.counters + p.K, sh.batch);
-  PHI_CUDA_TRY(cudaGetLastError());
-  return PHI_OK;
-}
-
-// The DDE convolution's boxes of n records.
-template <typename T, typename C>
-int launch_box_series(Plan& p, int g, const VisRec<T>* recs, int64_t n, C* boxes, int jmax,
-                      cudaStream_t s) {
-  SeriesShape sh;
-  PHI_TRY_ST((series_shape<T, C>(p, dde_box_series_kernel<T, C>, n, sh)));
-  dde_box_series_kernel<T, C><<<sh.blocks, 32 * sh.warps, sh.smem, s>>>(
-      recs, n, boxes, jmax, p.quad(), series_view<T, C>(p, g), p.counters + g, p.counters + p.K,
-      sh.batch);
   PHI_CUDA_TRY(cudaGetLastError());
   return PHI_OK;
 }
