@@ -6,7 +6,8 @@
 //                       fractional grid position, integer base, w offset,
 //                       weight and support;
 //   perm[n_kept]        caller index of each sorted record, bit 31 = folded;
-//   omn_pix[N*N]        1 - n(l, m) per pixel (FP64, for the chirp phase);
+//   omn_pix[N*N]        1 - n(l, m) per pixel, for the chirp phase (FP32: the
+//                       sum of two floats, 48 bits; FP64: a double);
 //   corr_pix[N*N]       1 / (g(du |l|) n(l, m)) per pixel (precision T);
 //   node tables         per panel count P = 1..128: 1 - n(r_j) (FP64) and
 //                       w 2 pi h g(r_j) r_j (T: the Kronrod weight, and the
@@ -174,7 +175,7 @@ struct Plan {
   // device memory
   void* recs = nullptr;
   uint32_t* perm = nullptr;
-  double* omn_pix = nullptr;
+  void* omn_pix = nullptr;   // float2 (FP32) or double (FP64)
   void* corr_pix = nullptr;
   double* node_omn = nullptr;
   float2* node_omn2 = nullptr;          // FP32: behind node_omn, in its allocation

@@ -238,6 +238,58 @@ __device__ double taper_g(double r, double a, double beta, double i0beta) {
   return 2.0 * kPi * a * a * f / i0beta;
 }
 
+// 1 - n as a sum of two floats (48 bits).
+__device__ __forceinline__ float2 two_floats(double v) {
+  const float hi = static_cast<float>(v);
+  return make_float2(hi, static_cast<float>(v - static_cast<double>(hi)));
+}
+// e^{2 pi i dw (1 - n)} in FP32: the phase from dw and 1 - n as sums of two
+// floats each, exact to 2^-48 of the product (the FP64 unit, at 1/64 of the
+// FP32 rate, would take longer than the work it serves).  FP64: directly.
+struct PhaseF {
+  float hi, lo;
+  __device__ __forceinline__ explicit PhaseF(double dw) {
+    hi = static_cast<float>(dw);
+    lo = static_cast<float>(dw - static_cast<double>(hi));
+  }
+  __device__ __forceinline__ float2 operator()(float omn_hi, float omn_lo) const {
+    const float p = __fmul_rn(hi, omn_hi);
+    float e = fmaf(hi, omn_hi, -p);
+    e = fmaf(hi, omn_lo, e);
+    e = fmaf(lo, omn_hi, e);
+    float sn, cs;
+    sincospif(2.0f * ((p - rintf(p)) + e), &sn, &cs);
+    return make_float2(cs, sn);
+  }
+};
+struct PhaseD {
+  double dw;
+  __device__ __forceinline__ explicit PhaseD(double w) : dw(w) {}
+  __device__ __forceinline__ double2 operator()(double omn) const {
+    double t = dw * omn;
+    t -= rint(t);
+    double sn, cs;
+    sincospi(2.0 * t, &sn, &cs);
+    return make_double2(cs, sn);
+  }
+};
+// 1 - n of a pixel as the tables hold it, and the phase that takes it.
+template <typename T> struct PixelPhase;
+template <> struct PixelPhase<float> {
+  typedef float2 omn;
+  PhaseF phase;
+  __device__ __forceinline__ explicit PixelPhase(double w) : phase(w) {}
+  __device__ __forceinline__ float2 operator()(float2 o) const { return phase(o.x, o.y); }
+  __device__ static __forceinline__ float2 make(double v) { return two_floats(v); }
+};
+template <> struct PixelPhase<double> {
+  typedef double omn;
+  PhaseD phase;
+  __device__ __forceinline__ explicit PixelPhase(double w) : phase(w) {}
+  __device__ __forceinline__ double2 operator()(double o) const { return phase(o); }
+  __device__ static __forceinline__ double make(double v) { return v; }
+};
+
 // ---------------------------------------------------------------------------
 // Tables built once per plan
 // ---------------------------------------------------------------------------
@@ -258,10 +310,7 @@ __global__ void node_table_kernel(double R, double du, double a, double beta, do
   double s = l * l;
   const double om = s / (1.0 + sqrt(1.0 - s));
   omn[j] = om;
-  if (omn2) {
-    const float hi = static_cast<float>(om);
-    omn2[j] = make_float2(hi, static_cast<float>(om - static_cast<double>(hi)));
-  }
+  if (omn2) omn2[j] = two_floats(om);
   double h = 2.0 * kPi * hw * taper_g(r, a, beta, cyl_bessel_i0(beta)) * r;
   hk[j] = static_cast<T>(gk_wk(k) * h);
   // FP32 quadrature forms its estimate from panel sums with the Gauss weight
@@ -271,14 +320,14 @@ __global__ void node_table_kernel(double R, double du, double a, double beta, do
 
 template <typename T>
 __global__ void pixel_table_kernel(int N, double dl, double du, double a, double beta,
-                                   double* omn, T* corr) {
+                                   typename PixelPhase<T>::omn* omn, T* corr) {
   int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= (int64_t)N * N) return;
   int row = static_cast<int>(idx / N), col = static_cast<int>(idx % N);
   double l = (col - N / 2) * dl, m = (row - N / 2) * dl;
   double s = l * l + m * m;
   double n = sqrt(1.0 - s);
-  omn[idx] = s / (1.0 + n);
+  omn[idx] = PixelPhase<T>::make(s / (1.0 + n));
   double g = taper_g(du * sqrt(s), a, beta, cyl_bessel_i0(beta));
   corr[idx] = static_cast<T>(1.0 / (g * n));
 }
@@ -304,10 +353,12 @@ int launch_pixel_tables(Plan& p, cudaStream_t s) {
   int blocks = static_cast<int>((total + 255) / 256);
   double a = 0.5 * p.d.support;
   if (p.d.precision == PHI_F64)
-    pixel_table_kernel<double><<<blocks, 256, 0, s>>>(p.N, p.dl, p.du, a, p.beta, p.omn_pix,
+    pixel_table_kernel<double><<<blocks, 256, 0, s>>>(p.N, p.dl, p.du, a, p.beta,
+                                                     static_cast<double*>(p.omn_pix),
                                                      static_cast<double*>(p.corr_pix));
   else
-    pixel_table_kernel<float><<<blocks, 256, 0, s>>>(p.N, p.dl, p.du, a, p.beta, p.omn_pix,
+    pixel_table_kernel<float><<<blocks, 256, 0, s>>>(p.N, p.dl, p.du, a, p.beta,
+                                                    static_cast<float2*>(p.omn_pix),
                                                     static_cast<float*>(p.corr_pix));
   PHI_CUDA_TRY(cudaGetLastError());
   return PHI_OK;
@@ -320,46 +371,60 @@ int launch_pixel_tables(Plan& p, cudaStream_t s) {
 // S~_k then Z for every stack of a group (blockIdx.y = slot): grid cell
 // (qv, qu) holds padded pixel P = (q + Npad/2) mod Npad (the centred image
 // moved to index 0), i.e. image pixel P - (Npad - N)/2, or zero outside.
+// Npad is even: a thread writes two neighbouring cells in one store.  Bound:
+// the grid's bytes (with FP64 phases the FP64 unit was).
 template <typename T, typename C>
-__global__ void prep_kernel(const T* __restrict__ x, const double* __restrict__ omn,
+__global__ void prep_kernel(const T* __restrict__ x,
+                            const typename PixelPhase<T>::omn* __restrict__ omn,
                             const T* __restrict__ corr, int N, int npad,
                             const double* __restrict__ wbar, const int32_t* __restrict__ stacks,
                             C* __restrict__ grids) {
+  struct __align__(2 * sizeof(C)) Pair { C c[2]; };
   const int off = (npad - N) / 2;
-  const double wb = wbar[stacks[blockIdx.y]];
+  const PixelPhase<T> phase(wbar[stacks[blockIdx.y]]);
   C* grid = grids + static_cast<int64_t>(blockIdx.y) * npad * npad;
   for (int qv = blockIdx.x; qv < npad; qv += gridDim.x) {
     int pv = qv + npad / 2;
     if (pv >= npad) pv -= npad;
     pv -= off;
     const bool row_in = pv >= 0 && pv < N;
-    for (int qu = threadIdx.x; qu < npad; qu += blockDim.x) {
-      int pu = qu + npad / 2;
-      if (pu >= npad) pu -= npad;
-      pu -= off;
-      C out = cmake<C>(0.0, 0.0);
-      if (row_in && pu >= 0 && pu < N) {
-        const int64_t pix = static_cast<int64_t>(pv) * N + pu;
-        double t = wb * omn[pix];
-        t -= rint(t);
-        T sn, cs;
-        sincos_pi(static_cast<T>(2.0 * t), &sn, &cs);
-        const T v = x[pix] * corr[pix];
-        out.x = v * cs;
-        out.y = v * sn;
+    for (int q0 = 2 * threadIdx.x; q0 < npad; q0 += 2 * blockDim.x) {
+      Pair out;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        int pu = q0 + k + npad / 2;
+        if (pu >= npad) pu -= npad;
+        pu -= off;
+        out.c[k] = cmake<C>(0.0, 0.0);
+        if (row_in && pu >= 0 && pu < N) {
+          const int64_t pix = static_cast<int64_t>(pv) * N + pu;
+          const C e = phase(omn[pix]);
+          const T v = x[pix] * corr[pix];
+          out.c[k].x = v * e.x;
+          out.c[k].y = v * e.y;
+        }
       }
-      grid[static_cast<int64_t>(qv) * npad + qu] = out;
+      *reinterpret_cast<Pair*>(grid + static_cast<int64_t>(qv) * npad + q0) = out;
     }
   }
 }
 
 // After the inverse FFTs of a group: x_p (+)= sum over its stacks of
-// Re(conj(S~_k) G_k[P(p)]), one pass over the image per group.
+// Re(conj(S~_k) G_k[P(p)]), one pass over the image per group.  The stacks'
+// centres are split into two floats once per block.  Bound: the grids' bytes
+// (with FP64 phases the FP64 unit was: 1.78 ms for 50 stacks of 2048^2).
+constexpr int kFinishStacks = 128;   // n_stacks is at most 126
 template <typename T, typename C>
-__global__ void finish_kernel(const C* __restrict__ grids, const double* __restrict__ omn,
+__global__ void finish_kernel(const C* __restrict__ grids,
+                              const typename PixelPhase<T>::omn* __restrict__ omn,
                               const T* __restrict__ corr, int N, int npad,
                               const double* __restrict__ wbar, const int32_t* __restrict__ stacks,
                               int nslots, T* __restrict__ x, int accumulate) {
+  __shared__ __align__(16) unsigned char phases_raw[kFinishStacks * sizeof(PixelPhase<T>)];
+  PixelPhase<T>* phases = reinterpret_cast<PixelPhase<T>*>(phases_raw);
+  for (int sl = threadIdx.x; sl < nslots; sl += blockDim.x)
+    phases[sl] = PixelPhase<T>(wbar[stacks[sl]]);
+  __syncthreads();
   const int off = (npad - N) / 2;
   const int64_t plane = static_cast<int64_t>(npad) * npad;
   for (int pv = blockIdx.x; pv < N; pv += gridDim.x) {
@@ -370,15 +435,13 @@ __global__ void finish_kernel(const C* __restrict__ grids, const double* __restr
       if (qu >= npad) qu -= npad;
       const int64_t pix = static_cast<int64_t>(pv) * N + pu;
       const int64_t gi = static_cast<int64_t>(qv) * npad + qu;
-      const double om = omn[pix];
+      const typename PixelPhase<T>::omn om = omn[pix];
       T acc = 0;
+#pragma unroll 4
       for (int sl = 0; sl < nslots; ++sl) {
         const C g = grids[sl * plane + gi];
-        double t = wbar[stacks[sl]] * om;
-        t -= rint(t);
-        T sn, cs;
-        sincos_pi(static_cast<T>(2.0 * t), &sn, &cs);
-        acc += cs * g.x + sn * g.y;
+        const C e = phases[sl](om);
+        acc += e.x * g.x + e.y * g.y;
       }
       const T v = corr[pix] * acc;
       x[pix] = accumulate ? x[pix] + v : v;
@@ -1464,26 +1527,6 @@ __global__ void __launch_bounds__(256) row_table_kernel(
   flush_counts(stats, 0, my_taps, 0, lane);
 }
 
-// e^{2 pi i dw (1 - n)} in FP32: the phase from dw and 1 - n as sums of two
-// floats each (48 bits; the FP64 unit, at 1/64 of the FP32 rate, would take
-// longer than the quadrature it serves).
-struct PhaseF {
-  float hi, lo;
-  __device__ __forceinline__ explicit PhaseF(double dw) {
-    hi = static_cast<float>(dw);
-    lo = static_cast<float>(dw - static_cast<double>(hi));
-  }
-  __device__ __forceinline__ float2 operator()(float omn_hi, float omn_lo) const {
-    const float p = __fmul_rn(hi, omn_hi);
-    float e = fmaf(hi, omn_hi, -p);
-    e = fmaf(hi, omn_lo, e);
-    e = fmaf(lo, omn_hi, e);
-    float sn, cs;
-    sincospif(2.0f * ((p - rintf(p)) + e), &sn, &cs);
-    return make_float2(cs, sn);
-  }
-};
-
 // [GC] at arbitrary points (phi_wkernel and phi_wkernel_noalloc): every point
 // has its own |dw|, so nothing but the node table is shared.  L lanes take a
 // point, each the nodes k = sub, sub + L, ... of every panel, with the node
@@ -2103,7 +2146,8 @@ int run_degrid(Plan& p, const T* x, C* y, cudaStream_t s, const DdeArgs* dde = n
     const int n = static_cast<int>(p.group_off[g + 1] - p.group_off[g]);
     ev = timer_begin(p, s);
     prep_kernel<T, C><<<dim3(p.num_sms * 4, n), 256, 0, s>>>(
-        x, p.omn_pix, static_cast<const T*>(p.corr_pix), p.N, p.npad, p.wbar_dev,
+        x, static_cast<const typename PixelPhase<T>::omn*>(p.omn_pix),
+        static_cast<const T*>(p.corr_pix), p.N, p.npad, p.wbar_dev,
         p.group_stacks_dev + p.group_off[g], grids);
     PHI_CUDA_TRY(cudaGetLastError());
     timer_end(p, ev, PHI_STAGE_PREP, s);
@@ -2180,7 +2224,8 @@ int run_grid(Plan& p, const C* y, T* x, cudaStream_t s, const DdeArgs* dde = nul
     timer_end(p, ev, PHI_STAGE_FFT, s);
     ev = timer_begin(p, s);
     finish_kernel<T, C><<<p.num_sms * 4, 256, 0, s>>>(
-        grids, p.omn_pix, static_cast<const T*>(p.corr_pix), p.N, p.npad, p.wbar_dev,
+        grids, static_cast<const typename PixelPhase<T>::omn*>(p.omn_pix),
+        static_cast<const T*>(p.corr_pix), p.N, p.npad, p.wbar_dev,
         p.group_stacks_dev + p.group_off[g], n, x, g == 0 ? 0 : 1);
     PHI_CUDA_TRY(cudaGetLastError());
     timer_end(p, ev, PHI_STAGE_FINISH, s);

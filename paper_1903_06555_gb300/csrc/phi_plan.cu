@@ -780,7 +780,8 @@ int build(Plan& p, const double* uvw, const double* weights, int64_t M, cudaStre
   PHI_CUDA_TRY(owned_alloc(p, reinterpret_cast<unsigned char**>(&p.node_hk), tsize * nodes));
   PHI_CUDA_TRY(owned_alloc(p, reinterpret_cast<unsigned char**>(&p.node_hd), tsize * nodes));
   PHI_TRY(build_tap_order(p, std::max(p.max_jw, 2), s));
-  PHI_CUDA_TRY(owned_alloc(p, &p.omn_pix, static_cast<size_t>(p.N) * p.N));
+  PHI_CUDA_TRY(owned_alloc(p, reinterpret_cast<double**>(&p.omn_pix),   // 8 bytes either way
+                           static_cast<size_t>(p.N) * p.N));
   PHI_CUDA_TRY(owned_alloc(p, reinterpret_cast<unsigned char**>(&p.corr_pix),
                            tsize * p.N * static_cast<size_t>(p.N)));
   PHI_CUDA_TRY(owned_alloc(p, &p.group_stacks_dev, std::max<size_t>(1, p.group_stacks.size())));
