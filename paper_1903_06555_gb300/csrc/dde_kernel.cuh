@@ -418,22 +418,37 @@ __global__ void __launch_bounds__(256) dde_conv_kernel(
 
 // The DDE convolution of the sampled quadrature (series_kernel.cuh): the taps
 // come cheaply from the visibility's polynomials, so the warp walks the box
-// in bands of four rows, kept in shared memory with the ring of row-pass rows
-// the column pass still needs: (a) the band's taps into `band`, 2 h zeros
-// either side of each row; (b) R(kb, cu) = sum_s a_s K(kb, cu - 2 h + s) of
-// its rows into ring row kb mod (4 + 2 h); (c) the combined rows cv = k0 ..
-// k0 + 3, C(cv, cu) = sum_s b_s R(cv - 2 h + s, cu), applied to the grid.
-// Rows outside the box are zeros in the ring.
+// in bands of four rows, kept in shared memory with the row-pass rows that
+// the column pass needs: (a) the band's taps, 2 h zeros either side of each
+// row; (b) R(kb, cu) = sum_s a_s K(kb, cu - 2 h + s) of its rows, behind the
+// 2 h rows of the band before; (c) the combined rows cv = k0 .. k0 + 3,
+// C(cv, cu) = sum_s b_s R(cv - 2 h + s, cu), applied to the grid; then the
+// last 2 h rows of R move to the front.  Rows outside the box are zeros.  A
+// lane takes two neighbouring rows of a column in (b) and (c), so that they
+// share the DDE's values, and in (c) all but one of the rows of R.
+//
+// Against boxes through global memory (dde_box_kernel's way, the boxes from
+// the polynomials): 5 x 5 kernels, 200,003 visibilities, J_w 24-42, one call:
+// 5.2 ms, and 7.9 with the buffer's first allocation; here 4.1, 1.7 of it this
+// kernel (2.6 there; 2.6 too with one row to a lane and a modular ring).
+// Bound: issue.
 constexpr int kDdeRows = 4;
-__host__ __device__ inline int dde_series_elems(int jmax, int jd) {
-  const int h2 = jd - 1;
-  return 2 * jd + kDdeRows * (jmax + 2 * h2) + (kDdeRows + h2) * (jmax + h2);
-}
-// acc + i acc2 accumulates a k as a.x k and a.y k apart.
-__device__ __forceinline__ void cmad_parts(float2& acc, float2& acc2, const float2& a,
+// A DDE value as the passes read it: FP32 both parts twice, for paired
+// arithmetic.
+template <typename C> struct DdeTap;
+template <> struct DdeTap<float2> {
+  typedef float4 type;
+  __device__ static __forceinline__ float4 make(const float2& a) { return make_float4(a.x, a.x, a.y, a.y); }
+};
+template <> struct DdeTap<double2> {
+  typedef double2 type;
+  __device__ static __forceinline__ double2 make(const double2& a) { return a; }
+};
+// acc += a.x k, acc2 += a.y k: acc + i acc2 accumulates a k.
+__device__ __forceinline__ void cmad_parts(float2& acc, float2& acc2, const float4& a,
                                            const float2& k) {
-  acc = __ffma2_rn(make_float2(a.x, a.x), k, acc);
-  acc2 = __ffma2_rn(make_float2(a.y, a.y), k, acc2);
+  acc = __ffma2_rn(make_float2(a.x, a.y), k, acc);
+  acc2 = __ffma2_rn(make_float2(a.z, a.w), k, acc2);
 }
 __device__ __forceinline__ void cmad_parts(double2& acc, double2& acc2, const double2& a,
                                            const double2& k) {
@@ -442,24 +457,41 @@ __device__ __forceinline__ void cmad_parts(double2& acc, double2& acc2, const do
   acc2.x = fma(a.y, k.x, acc2.x);
   acc2.y = fma(a.y, k.y, acc2.y);
 }
-template <typename T, typename C, bool kGrid>
+template <typename C>
+__device__ __forceinline__ C cmad_sum(const C& acc, const C& acc2) {
+  C r;
+  r.x = acc.x - acc2.y;
+  r.y = acc.y + acc2.x;
+  return r;
+}
+// Bytes of one warp beside the series: the DDE's values, the band, the rows of R.
+template <typename C>
+__host__ __device__ inline int dde_series_bytes(int jmax, int jd) {
+  const int h2 = jd - 1;
+  return 2 * jd * 16 + static_cast<int>(sizeof(C)) *
+                           (kDdeRows * (jmax + 2 * h2) + (kDdeRows + h2) * (jmax + h2));
+}
+// kJd: the DDE's taps a side when known at compile time (0: any).
+template <typename T, typename C, bool kGrid, int kJd>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) dde_series_kernel(
     const VisRec<T>* __restrict__ recs, const uint32_t* __restrict__ perm, int64_t n,
     const C* __restrict__ grid_in, C* grid_out, const C* __restrict__ vis_in,
     C* __restrict__ vis_out, QuadParams q, SeriesView<T> sv, const C* __restrict__ dde_a,
-    const C* __restrict__ dde_b, int jd, int jmax, const int32_t* __restrict__ stack_slot,
+    const C* __restrict__ dde_b, int jd_any, int jmax, const int32_t* __restrict__ stack_slot,
     unsigned long long* head, unsigned long long* stats, int batch) {
+  typedef typename DdeTap<C>::type Tap;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
+  const int jd = kJd ? kJd : jd_any;
   const int series_bytes = series_warp_bytes<T>(sv.stride, sv.max_intervals);
-  unsigned char* base = smem_raw + (threadIdx.x >> 5) *
-                        (series_bytes + dde_series_elems(jmax, jd) * static_cast<int>(sizeof(C)));
+  unsigned char* base =
+      smem_raw + (threadIdx.x >> 5) * (series_bytes + dde_series_bytes<C>(jmax, jd));
   SeriesWarp<T, C> w(base, sv);
-  const int h = jd >> 1, h2 = 2 * h, nring = kDdeRows + h2;
-  const int bw = jmax + 2 * h2, rw = jmax + h2;   // row lengths of the band and the ring
-  C* dab = reinterpret_cast<C*>(base + series_bytes);   // a_i then b_i
-  C* band = dab + 2 * jd;
-  C* ring = band + kDdeRows * bw;
+  const int h = jd >> 1, h2 = 2 * h;
+  const int bw = jmax + 2 * h2, rw = jmax + h2;   // row lengths of the band and of R
+  Tap* dab = reinterpret_cast<Tap*>(base + series_bytes);   // a_i then b_i
+  C* band = reinterpret_cast<C*>(dab + 2 * jd);
+  C* R = band + kDdeRows * bw;
   unsigned long long my_taps = 0, my_nodes = 0;
   const int npad = q.npad;
   const C zero = cmake<C>(0.0, 0.0);
@@ -480,18 +512,17 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) dde_series_kernel
       const int64_t src = pm & 0x7fffffffu;
       const C yv = kGrid ? load_visibility<T, C>(vis_in, pm, static_cast<T>(r.weight)) : zero;
       if (lane < 2 * jd)
-        dab[lane] = lane < jd ? dde_a[src * jd + lane] : dde_b[src * jd + lane - jd];
-      for (int e = lane; e < kDdeRows * h2; e += 32) {   // the band's zeros, 2 h to a side
-        const int row = e / h2, s = e - row * h2;
-        band[row * bw + s] = zero;
-        band[row * bw + h2 + Jw + s] = zero;
-      }
-      for (int e = lane; e < nring * rw; e += 32) ring[e] = zero;
+        dab[lane] = DdeTap<C>::make(lane < jd ? dde_a[src * jd + lane] : dde_b[src * jd + lane - jd]);
+      for (int s = lane; s < h2; s += 32)            // the band's zeros, 2 h to a side
+#pragma unroll
+        for (int row = 0; row < kDdeRows; ++row)
+          band[row * bw + s] = band[row * bw + h2 + Jw + s] = zero;
+      for (int cu = lane; cu < Jc; cu += 32)
+        for (int row = 0; row < h2; ++row) R[row * rw + cu] = zero;
       C accv = zero;
-      // box origin on the grid; columns and rows wrap by one conditional
-      const int u0 = r.bu - h - half + 1, v0 = r.bv - h - half + 1;
-      const int step_r = 32 / Jc, step_c = 32 % Jc;
-      int slot0 = nring - h2;                            // ring row of kb = k0 - 2 h
+      const int u0 = wrap_index(r.bu - h - half + 1, npad);
+      const int v0 = wrap_index(r.bv - h - half + 1, npad);
+      const bool contig = u0 + Jc <= npad && v0 + Jc <= npad;
       for (int k0 = 0; k0 < Jc; k0 += kDdeRows) {
         __syncwarp();
         // (a) the taps of rows k0 .. k0 + 3; rows past the box are zeros
@@ -499,14 +530,18 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) dde_series_kernel
           const int row = 2 * ((lane >> 3) & 1);
           const float nb = static_cast<float>(half - 1 - k0 - row);
           const float2 dv_ = __fadd2_rn(make_float2(r.fv, r.fv), make_float2(nb, nb - 1.0f));
-          for (int a = (lane & 7) | ((lane & 16) >> 1); a < Jw; a += 16) {
-            const float du_ = r.fu + static_cast<float>(half - 1 - a), d2 = du_ * du_;
+          const bool in = k0 + row < Jw;
+          int c = (lane & 7) | ((lane & 16) >> 1);
+          float na = static_cast<float>(half - 1 - c);
+          C* out = band + row * bw + h2 + c;
+          for (; c < Jw; c += 16, na -= 16.0f, out += 16) {
+            const float du_ = r.fu + na, d2 = du_ * du_;
             float2 t0 = zero, t1 = zero;
-            if (k0 + row < Jw)
+            if (in)
               series_eval2(w.coef, w.slots, sv.inv_delta,
                            __ffma2_rn(dv_, dv_, make_float2(d2, d2)), t0, t1);
-            band[row * bw + h2 + a] = t0;
-            band[(row + 1) * bw + h2 + a] = t1;
+            out[0] = t0;
+            out[bw] = t1;
           }
         } else {
           for (int e = lane; e < kDdeRows * Jw; e += 32) {
@@ -519,56 +554,58 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) dde_series_kernel
           }
         }
         __syncwarp();
-        // (b) their rows of R; slot1: the ring row of kb = k0
-        int slot1 = slot0 + h2;
-        if (slot1 >= nring) slot1 -= nring;
-        for (int rr = lane / Jc, cu = lane - rr * Jc; rr < kDdeRows;) {
+        // (b) their rows of R, two to a lane
+        for (int x = lane; x < 2 * Jc; x += 32) {
+          const int cu = x < Jc ? x : x - Jc, rr = x < Jc ? 0 : 2;
           const C* k = band + rr * bw + cu;
-          C acc = zero, acc2 = zero;
-#pragma unroll 5
-          for (int s = 0; s < jd; ++s) cmad_parts(acc, acc2, dab[s], k[s]);
-          int sl = slot1 + rr;
-          if (sl >= nring) sl -= nring;
-          acc.x -= acc2.y;
-          acc.y += acc2.x;
-          ring[sl * rw + cu] = acc;
-          rr += step_r;
-          cu += step_c;
-          if (cu >= Jc) {
-            cu -= Jc;
-            ++rr;
+          C p0 = zero, q0 = zero, p1 = zero, q1 = zero;
+#pragma unroll
+          for (int s = 0; s < (kJd ? kJd : 15); ++s) {
+            if (!kJd && s >= jd) break;
+            const Tap a = dab[s];
+            cmad_parts(p0, q0, a, k[s]);
+            cmad_parts(p1, q1, a, k[bw + s]);
           }
+          R[(h2 + rr) * rw + cu] = cmad_sum(p0, q0);
+          R[(h2 + rr + 1) * rw + cu] = cmad_sum(p1, q1);
         }
         __syncwarp();
-        // (c) the combined rows k0 .. k0 + 3
-        for (int rr = lane / Jc, cu = lane - rr * Jc; rr < kDdeRows && k0 + rr < Jc;) {
-          C acc = zero, acc2 = zero;
-          int sl = slot0 + rr;
-          if (sl >= nring) sl -= nring;
-#pragma unroll 5
-          for (int s = 0; s < jd; ++s) {
-            cmad_parts(acc, acc2, dab[jd + s], ring[sl * rw + cu]);
-            sl = sl + 1 == nring ? 0 : sl + 1;
+        // (c) the combined rows k0 .. k0 + 3 (an even number: J_w + 2 h is)
+        for (int x = lane; x < 2 * Jc; x += 32) {
+          const int cu = x < Jc ? x : x - Jc, rr = x < Jc ? 0 : 2;
+          if (k0 + rr >= Jc) break;
+          const C* rows = R + rr * rw + cu;
+          C p0 = zero, q0 = zero, p1 = zero, q1 = zero, row = rows[0];
+#pragma unroll
+          for (int s = 0; s < (kJd ? kJd : 15); ++s) {
+            if (!kJd && s >= jd) break;
+            const Tap b = dab[jd + s];
+            cmad_parts(p0, q0, b, row);
+            rows += rw;
+            row = rows[0];
+            cmad_parts(p1, q1, b, row);
           }
-          acc.x -= acc2.y;
-          acc.y += acc2.x;
-          ++my_taps;
-          apply_tap<C, kGrid>(acc, gbase + static_cast<int64_t>(wrap_index(v0 + k0 + rr, npad)) * npad +
-                                       wrap_index(u0 + cu, npad),
-                              yv, grid_in, grid_out, q.fx, accv);
-          rr += step_r;
-          cu += step_c;
-          if (cu >= Jc) {
-            cu -= Jc;
-            ++rr;
+          my_taps += 2;
+          int64_t g0, g1;
+          if (contig) {
+            g0 = gbase + static_cast<int64_t>(v0 + k0 + rr) * npad + u0 + cu;
+            g1 = g0 + npad;
+          } else {
+            const int64_t col = gbase + wrap_index(u0 + cu, npad);
+            g0 = col + static_cast<int64_t>(wrap_index(v0 + k0 + rr, npad)) * npad;
+            g1 = col + static_cast<int64_t>(wrap_index(v0 + k0 + rr + 1, npad)) * npad;
           }
+          apply_tap<C, kGrid>(cmad_sum(p0, q0), g0, yv, grid_in, grid_out, q.fx, accv);
+          apply_tap<C, kGrid>(cmad_sum(p1, q1), g1, yv, grid_in, grid_out, q.fx, accv);
         }
-        slot0 += kDdeRows;
-        if (slot0 >= nring) slot0 -= nring;
+        __syncwarp();
+        // the last 2 h rows of R to the front, each lane its own columns
+        for (int cu = lane; cu < Jc; cu += 32)
+          for (int row = 0; row < h2; ++row) R[row * rw + cu] = R[(row + kDdeRows) * rw + cu];
       }
       if (lane == 0) my_nodes += static_cast<unsigned long long>((NP + 1) * kNodes * P);
       if (!kGrid) store_visibility<T, C>(accv, static_cast<T>(r.weight), pm, vis_out, lane);
-      __syncwarp();   // the polynomials, the band and the ring are rewritten
+      __syncwarp();   // the polynomials, the band and R are rewritten
     }
   }
   flush_counts(stats, 0, my_taps, my_nodes, lane);

@@ -117,12 +117,17 @@ int launch_dde_series(Plan& p, int g, const VisRec<T>* recs, int64_t b0, int64_t
                       const C* grids_in, C* grids_out, const C* vis_in, C* vis_out,
                       const DdeArgs& dde, cudaStream_t s, bool& launched) {
   const int jmax = std::max(p.max_jw, 2);
-  const size_t extra = sizeof(C) * static_cast<size_t>(dde_series_elems(jmax, dde.jd));
+  const size_t extra = static_cast<size_t>(dde_series_bytes<C>(jmax, dde.jd));
+  // the usual small kernels unrolled, any other in a loop
+  auto kernel = dde.jd == 3   ? dde_series_kernel<T, C, kGrid, 3>
+                : dde.jd == 5 ? dde_series_kernel<T, C, kGrid, 5>
+                : dde.jd == 7 ? dde_series_kernel<T, C, kGrid, 7>
+                              : dde_series_kernel<T, C, kGrid, 0>;
   SeriesShape sh;
-  PHI_TRY_ST((series_shape<T, C>(p, dde_series_kernel<T, C, kGrid>, nk, extra, sh)));
+  PHI_TRY_ST((series_shape<T, C>(p, kernel, nk, extra, sh)));
   launched = sh.warps > 0;
   if (!launched) return PHI_OK;
-  dde_series_kernel<T, C, kGrid><<<sh.blocks, 32 * sh.warps, sh.smem, s>>>(
+  kernel<<<sh.blocks, 32 * sh.warps, sh.smem, s>>>(
       recs, p.perm + b0, nk, grids_in, grids_out, vis_in, vis_out, p.quad(),
       series_view<T, C>(p, g), static_cast<const C*>(dde.a), static_cast<const C*>(dde.b), dde.jd,
       jmax, p.stack_slot_dev, p.counters + g, p.counters + p.K, sh.batch);

@@ -2303,13 +2303,23 @@ void timer_end(Plan& p, long idx, int stage, cudaStream_t s) {
   p.ev_pending.emplace_back(stage, static_cast<size_t>(idx));
 }
 
+template <typename T, typename C, int kJd>
+cudaError_t set_dde_series_smem(int bytes) {
+  const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(dde_series_kernel<T, C, false, kJd>, a, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(dde_series_kernel<T, C, true, kJd>, a, bytes);
+  return e;
+}
+
 template <typename T, typename C>
 cudaError_t set_series_smem(int bytes) {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaFuncSetAttribute(vis_series_kernel<T, C, false>, a, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(vis_series_kernel<T, C, true>, a, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(dde_series_kernel<T, C, false>, a, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(dde_series_kernel<T, C, true>, a, bytes);
+  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 0>(bytes);
+  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 3>(bytes);
+  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 5>(bytes);
+  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 7>(bytes);
   return e;
 }
 
