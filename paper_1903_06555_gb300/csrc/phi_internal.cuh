@@ -190,7 +190,8 @@ struct Plan {
   int32_t* group_stacks_dev = nullptr;
   int32_t* stack_slot_dev = nullptr;    // slot of each stack within its group
   double* wbar_dev = nullptr;
-  cufftHandle fft_batch = 0;            // `group` transforms in one call
+  cufftHandle fft_batch = 0;            // fft_batch_n transforms in one call
+  int fft_batch_n = 1;
   bool fft_batch_ok = false;
   // [0..K) work heads, [K] unconverged taps, [K+1] taps, [K+2] wkernel misses,
   // [K+3] tap-node evaluations; retry_counters[2 g], [2 g + 1], g < K: length

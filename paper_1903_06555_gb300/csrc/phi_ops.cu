@@ -2028,8 +2028,8 @@ int launch_row_table(Plan& p, int g, const C* grids_in, C* grids_out, const C* v
   return PHI_OK;
 }
 
-// In-place FFTs of the first n grids of the group (one batched call when
-// the group is full).
+// In-place FFTs of the first n grids of the group, fft_batch_n to a call and
+// the rest one by one.
 template <typename T, typename C>
 int fft_group(Plan& p, C* grids, int n, int dir, cudaStream_t s) {
   const int64_t plane = static_cast<int64_t>(p.npad) * p.npad;
@@ -2041,12 +2041,12 @@ int fft_group(Plan& p, C* grids, int n, int dir, cudaStream_t s) {
     return cufftExecC2C(h, reinterpret_cast<cufftComplex*>(g), reinterpret_cast<cufftComplex*>(g),
                         dir);
   };
-  if (n == p.group && p.fft_batch_ok) {
-    if (run(p.fft_batch, grids) != CUFFT_SUCCESS) return PHI_ERR_CUDA;
-  } else {
-    for (int i = 0; i < n; ++i)
-      if (run(p.fft, grids + i * plane) != CUFFT_SUCCESS) return PHI_ERR_CUDA;
-  }
+  int i = 0;
+  if (p.fft_batch_ok)
+    for (; i + p.fft_batch_n <= n; i += p.fft_batch_n)
+      if (run(p.fft_batch, grids + i * plane) != CUFFT_SUCCESS) return PHI_ERR_CUDA;
+  for (; i < n; ++i)
+    if (run(p.fft, grids + i * plane) != CUFFT_SUCCESS) return PHI_ERR_CUDA;
   return PHI_OK;
 }
 
