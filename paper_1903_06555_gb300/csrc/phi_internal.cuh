@@ -192,6 +192,8 @@ struct Plan {
   double* wbar_dev = nullptr;
   cufftHandle fft_batch = 0;            // fft_batch_n transforms in one call
   int fft_batch_n = 1;
+  int fft_log = 0;                      // two-pass transforms: log2 N (0: cuFFT)
+  void* fft_tab = nullptr;              // their roots of unity
   bool fft_batch_ok = false;
   // [0..K) work heads, [K] unconverged taps, [K+1] taps, [K+2] wkernel misses,
   // [K+3] tap-node evaluations; retry_counters[2 g], [2 g + 1], g < K: length
@@ -310,6 +312,9 @@ int launch_pixel_tables(Plan& p, cudaStream_t s);
 int build_kernel_table(Plan& p, cudaStream_t s);
 int build_radial_tables(Plan& p, cudaStream_t s);
 int build_series_tables(Plan& p, cudaStream_t s);
+int fft_two_pass_log(int N, int npad, bool f64);   // log2 N where the two-pass transforms apply, or 0
+int fft_two_pass_table(int N);           // complex values of their table
+int build_fft_table(Plan& p, cudaStream_t s);
 int compute_kernel_bound(Plan& p, double* scratch, cudaStream_t s);  // scratch: kMaxPanels doubles
 
 }  // namespace phi

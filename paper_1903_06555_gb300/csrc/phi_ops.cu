@@ -483,6 +483,9 @@ __global__ void finish_kernel(const C* __restrict__ grids,
   }
 }
 
+// The image-domain steps and the FFTs in two passes, for N = 2^6 .. 2^11, os 2
+#include "fft_kernel.cuh"
+
 // ---------------------------------------------------------------------------
 // Deterministic gridding: fixed-point grid sums
 // ---------------------------------------------------------------------------
@@ -2093,6 +2096,9 @@ struct DdeArgs {
   int jd;
 };
 
+// launch_fft_forward, launch_fft_adjoint
+#include "fft_launch.cuh"
+
 // launch_series, dde_warp_smem, launch_dde
 #include "series_launch.cuh"
 #include "dde_launch.cuh"
@@ -2168,6 +2174,54 @@ int launch_group_kernel(Plan& p, int g, const C* grids_in, C* grids_out, const C
   return PHI_OK;
 }
 
+// S~_k, Z and F for the n grids of group g: the two-pass transforms where
+// they take the grid (the row pass timed as prep, the column pass as FFT),
+// prep and cuFFT otherwise.
+template <typename T, typename C>
+int image_to_grids(Plan& p, int g, int n, const T* x, C* grids, cudaStream_t s) {
+  const int32_t* stacks = p.group_stacks_dev + p.group_off[g];
+  long ev = timer_begin(p, s);
+  if (p.fft_log) {
+    PHI_TRY_ST((fft_pass<T, C>(p, kFftRowsForward, stacks, n, x, grids, nullptr, 0, s)));
+  } else {
+    prep_kernel<T, C><<<dim3(p.num_sms * 4, n), 256, 0, s>>>(
+        x, static_cast<const typename PixelPhase<T>::omn*>(p.omn_pix),
+        static_cast<const T*>(p.corr_pix), p.N, p.npad, p.wbar_dev, stacks, grids);
+    PHI_CUDA_TRY(cudaGetLastError());
+  }
+  timer_end(p, ev, PHI_STAGE_PREP, s);
+  ev = timer_begin(p, s);
+  if (p.fft_log)
+    PHI_TRY_ST((fft_pass<T, C>(p, kFftColsForward, stacks, n, x, grids, nullptr, 0, s)));
+  else
+    PHI_TRY_ST((fft_group<T, C>(p, grids, n, CUFFT_FORWARD, s)));
+  timer_end(p, ev, PHI_STAGE_FFT, s);
+  return PHI_OK;
+}
+
+// F^H, Z^T and conj(S~_k), summed into the image.
+template <typename T, typename C>
+int grids_to_image(Plan& p, int g, int n, C* grids, T* x, cudaStream_t s) {
+  const int32_t* stacks = p.group_stacks_dev + p.group_off[g];
+  long ev = timer_begin(p, s);
+  if (p.fft_log)
+    PHI_TRY_ST((fft_pass<T, C>(p, kFftColsAdjoint, stacks, n, nullptr, grids, nullptr, 0, s)));
+  else
+    PHI_TRY_ST((fft_group<T, C>(p, grids, n, CUFFT_INVERSE, s)));
+  timer_end(p, ev, PHI_STAGE_FFT, s);
+  ev = timer_begin(p, s);
+  if (p.fft_log) {
+    PHI_TRY_ST((fft_pass<T, C>(p, kFftRowsAdjoint, stacks, n, nullptr, grids, x, g == 0 ? 0 : 1, s)));
+  } else {
+    finish_kernel<T, C><<<p.num_sms * 4, 256, 0, s>>>(
+        grids, static_cast<const typename PixelPhase<T>::omn*>(p.omn_pix),
+        static_cast<const T*>(p.corr_pix), p.N, p.npad, p.wbar_dev, stacks, n, x, g == 0 ? 0 : 1);
+    PHI_CUDA_TRY(cudaGetLastError());
+  }
+  timer_end(p, ev, PHI_STAGE_FINISH, s);
+  return PHI_OK;
+}
+
 template <typename T, typename C>
 int run_degrid(Plan& p, const T* x, C* y, cudaStream_t s, const DdeArgs* dde = nullptr) {
   long ev = timer_begin(p, s);
@@ -2178,16 +2232,7 @@ int run_degrid(Plan& p, const T* x, C* y, cudaStream_t s, const DdeArgs* dde = n
   const int ngroups = static_cast<int>(p.group_off.size()) - 1;
   for (int g = 0; g < ngroups; ++g) {
     const int n = static_cast<int>(p.group_off[g + 1] - p.group_off[g]);
-    ev = timer_begin(p, s);
-    prep_kernel<T, C><<<dim3(p.num_sms * 4, n), 256, 0, s>>>(
-        x, static_cast<const typename PixelPhase<T>::omn*>(p.omn_pix),
-        static_cast<const T*>(p.corr_pix), p.N, p.npad, p.wbar_dev,
-        p.group_stacks_dev + p.group_off[g], grids);
-    PHI_CUDA_TRY(cudaGetLastError());
-    timer_end(p, ev, PHI_STAGE_PREP, s);
-    ev = timer_begin(p, s);
-    PHI_TRY_ST((fft_group<T, C>(p, grids, n, CUFFT_FORWARD, s)));
-    timer_end(p, ev, PHI_STAGE_FFT, s);
+    PHI_TRY_ST((image_to_grids<T, C>(p, g, n, x, grids, s)));
     ev = timer_begin(p, s);
     PHI_TRY_ST((launch_group_kernel<T, C, false>(p, g, grids, nullptr, nullptr, y, s, dde)));
     timer_end(p, ev, PHI_STAGE_DEGRID, s);
@@ -2253,16 +2298,7 @@ int run_grid(Plan& p, const C* y, T* x, cudaStream_t s, const DdeArgs* dde = nul
       PHI_CUDA_TRY(cudaGetLastError());
     }
     timer_end(p, ev, PHI_STAGE_GRID, s);
-    ev = timer_begin(p, s);
-    PHI_TRY_ST((fft_group<T, C>(p, grids, n, CUFFT_INVERSE, s)));
-    timer_end(p, ev, PHI_STAGE_FFT, s);
-    ev = timer_begin(p, s);
-    finish_kernel<T, C><<<p.num_sms * 4, 256, 0, s>>>(
-        grids, static_cast<const typename PixelPhase<T>::omn*>(p.omn_pix),
-        static_cast<const T*>(p.corr_pix), p.N, p.npad, p.wbar_dev,
-        p.group_stacks_dev + p.group_off[g], n, x, g == 0 ? 0 : 1);
-    PHI_CUDA_TRY(cudaGetLastError());
-    timer_end(p, ev, PHI_STAGE_FINISH, s);
+    PHI_TRY_ST((grids_to_image<T, C>(p, g, n, grids, x, s)));
   }
   if (ngroups == 0) PHI_CUDA_TRY(cudaMemsetAsync(x, 0, sizeof(T) * (size_t)p.N * p.N, s));
   return PHI_OK;
@@ -2295,6 +2331,21 @@ int build_kernel_table(Plan& p, cudaStream_t s) {
 int build_radial_tables(Plan& p, cudaStream_t s) {
   if (p.d.precision == PHI_F64) return build_radial_tables_t<double, double2>(p, s);
   return build_radial_tables_t<float, float2>(p, s);
+}
+
+int fft_two_pass_log(int N, int npad, bool f64) { return fft_log(N, npad, f64); }
+int fft_two_pass_table(int N) { return fft_table_size(N); }
+
+int build_fft_table(Plan& p, cudaStream_t s) {
+  const int blocks = (fft_table_size(p.N) + 255) / 256;
+  if (p.d.precision == PHI_F64)
+    fft_table_kernel<double, double2><<<blocks, 256, 0, s>>>(p.fft_log,
+                                                             static_cast<double2*>(p.fft_tab));
+  else
+    fft_table_kernel<float, float2><<<blocks, 256, 0, s>>>(p.fft_log,
+                                                           static_cast<float2*>(p.fft_tab));
+  PHI_CUDA_TRY(cudaGetLastError());
+  return PHI_OK;
 }
 
 int build_series_tables(Plan& p, cudaStream_t s) {
@@ -2415,6 +2466,8 @@ int set_kernel_smem_limits() {
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
   PHI_CUDA_TRY(cudaFuncSetAttribute(vis_radial_kernel<double, double2, true>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
+  PHI_TRY_ST((set_fft_smem<float, float2>()));
+  PHI_TRY_ST((set_fft_smem<double, double2>()));
   PHI_CUDA_TRY((set_series_smem<float, float2>(optin)));
   PHI_CUDA_TRY((set_series_smem<double, double2>(optin)));
   PHI_CUDA_TRY((set_dde_smem<float, float2>(optin)));

@@ -341,6 +341,7 @@ void free_plan(Plan* p) {
   cudaFree(p->radial_tab);
   cudaFree(p->grid);
   cudaFree(p->retry_counters);
+  cudaFree(p->fft_tab);
   cudaFree(p->series_j0);
   cudaFree(p->series_nodes);
   cudaFree(p->retry);
@@ -821,6 +822,14 @@ int build(Plan& p, const double* uvw, const double* weights, int64_t M, cudaStre
   }
   if (d.kernel_mode == PHI_KERNEL_RADIAL) PHI_TRY(build_radial_tables(p, s));
   if (d.kernel_mode != PHI_KERNEL_TABLE) PHI_TRY(build_series_tables(p, s));
+  p.fft_log = fft_two_pass_log(p.N, p.npad, f64);
+  if (p.fft_log) {
+    PHI_CUDA_TRY(owned_alloc(p, reinterpret_cast<unsigned char**>(&p.fft_tab),
+                             2 * tsize * static_cast<size_t>(fft_two_pass_table(p.N))));
+    PHI_TRY(build_fft_table(p, s));
+    PHI_CUDA_TRY(cudaStreamSynchronize(s));
+    return PHI_OK;
+  }
   if (cufftCreate(&p.fft) != CUFFT_SUCCESS) return PHI_ERR_CUDA;
   p.fft_ok = true;
   size_t work = 0;
