@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) vis_dde_kernel(
     C* __restrict__ vis_out, QuadParams q, RadialView<T> rv, const C* __restrict__ dde_a,
     const C* __restrict__ dde_b, int jd, int jmax, const int32_t* __restrict__ stack_slot,
     unsigned long long* head, unsigned long long* stats, int batch, RecordList list) {
+  if (list.empty()) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;

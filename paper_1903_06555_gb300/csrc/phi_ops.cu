@@ -1015,6 +1015,9 @@ struct RecordList {
   __device__ __forceinline__ unsigned long long record(unsigned long long i) const {
     return index ? index[i] : i;
   }
+  // As a rule: nothing was left to the list, and every warp of the launch
+  // would ask the queue's head in vain (6.6 us; 2.2 us with this test).
+  __device__ __forceinline__ bool empty() const { return index && *n == 0; }
 };
 
 // The value a gridded visibility spreads: W_i y_i, conjugated back if folded.
@@ -1108,6 +1111,7 @@ __global__ void __launch_bounds__(VisLaunch<T>::threads, VisLaunch<T>::min_block
                const C* __restrict__ grid_in, C* grid_out, const C* __restrict__ vis_in,
                C* __restrict__ vis_out, QuadParams q, const int32_t* __restrict__ stack_slot,
                unsigned long long* head, unsigned long long* stats, int batch, RecordList list) {
+  if (list.empty()) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -1805,6 +1809,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) vis_radial_kernel
     C* __restrict__ vis_out, QuadParams q, RadialView<T> rv,
     const int32_t* __restrict__ stack_slot, unsigned long long* head,
     unsigned long long* stats, int batch, RecordList list) {
+  if (list.empty()) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -2225,7 +2230,7 @@ int grids_to_image(Plan& p, int g, int n, C* grids, T* x, cudaStream_t s) {
 template <typename T, typename C>
 int run_degrid(Plan& p, const T* x, C* y, cudaStream_t s, const DdeArgs* dde = nullptr) {
   long ev = timer_begin(p, s);
-  PHI_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(C) * (size_t)p.M, s));
+  if (p.n_dropped > 0) PHI_CUDA_TRY(cudaMemsetAsync(y, 0, sizeof(C) * (size_t)p.M, s));
   PHI_CUDA_TRY(cudaMemsetAsync(p.retry_counters, 0, sizeof(unsigned long long) * 3 * p.K, s));
   timer_end(p, ev, PHI_STAGE_CLEAR, s);
   C* grids = static_cast<C*>(p.grid);
