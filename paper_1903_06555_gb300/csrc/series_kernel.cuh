@@ -378,27 +378,26 @@ __device__ __forceinline__ void series_polynomials(const float2* smp, float2* co
   }
   __syncwarp();
 }
+// (FP64: a lane takes the real or the imaginary part of an interval, so that
+// fewer lanes of its FP64 unit idle in the last round.)
 __device__ __forceinline__ void series_polynomials(const double2* smp, double2* coef, int slots,
                                                    int NP, int lane) {
   constexpr int H = SeriesN<double>::half, M = SeriesN<double>::terms;
-  for (int p = lane; p < NP; p += 32) {
-    double2 c[M];
+  const double* part = reinterpret_cast<const double*>(smp) + (lane & 1);
+  double* out = reinterpret_cast<double*>(coef) + (lane & 1);
+  for (int p = lane >> 1; p < NP; p += 16) {
+    double c[M];
 #pragma unroll
-    for (int m = 0; m < M; ++m) c[m] = make_double2(0.0, 0.0);
-#pragma unroll 2
+    for (int m = 0; m < M; ++m) c[m] = 0.0;
+#pragma unroll 4
     for (int d = 0; d < H; ++d) {
-      const double2 lo = smp[abs(p - d)], hi = smp[p + 1 + d];
-      const double2 sum = make_double2(hi.x + lo.x, hi.y + lo.y);
-      const double2 dif = make_double2(hi.x - lo.x, hi.y - lo.y);
+      const double lo = part[2 * abs(p - d)], hi = part[2 * (p + 1 + d)];
+      const double sum = hi + lo, dif = hi - lo;
 #pragma unroll
-      for (int m = 0; m < M; ++m) {
-        const double2 f = (m & 1) ? dif : sum;
-        c[m].x = fma(c_series_d[m][d], f.x, c[m].x);
-        c[m].y = fma(c_series_d[m][d], f.y, c[m].y);
-      }
+      for (int m = 0; m < M; ++m) c[m] = fma(c_series_d[m][d], (m & 1) ? dif : sum, c[m]);
     }
 #pragma unroll
-    for (int k = 0; k < M; ++k) coef[k * slots + series_slot(p)] = c[k];
+    for (int m = 0; m < M; ++m) out[2 * (m * slots + series_slot(p))] = c[m];
   }
   __syncwarp();
 }
