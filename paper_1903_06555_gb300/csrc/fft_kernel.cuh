@@ -16,14 +16,15 @@
 // N, the row pass transforms them, applies conj(S~_k), sums over the group's
 // stacks and writes the image.  Against separate steps around a library FFT
 // the zero half is neither written, transformed nor read: 2 N^2 grid values
-// of 8 bytes in and out per stack and direction in place of 5 of prep (write)
-// and the FFT's two passes: 8 stacks of 4096^2 in
-// FP32, forward 0.73 ms (prep 0.24 and cuFFT 1.01), adjoint 0.73 ms (cuFFT
-// 1.03 and the image step 0.11), and no library workspace (1 GiB).  Bound: the
-// column passes by the latency of their exchanges (16 warps per SM; 3 TB/s),
-// the row passes by shared memory (75%).  Tried for the column passes:
-// persistent blocks with the next tile by cp.async (0.54 and 0.60 ms against
-// 0.53), 2 columns in place of 4 (0.73), 64 registers (0.83, spills).
+// in and out per stack and direction, where the image step's write and the
+// library's two passes over the padded grid moved 5 times that.  8 stacks of
+// 4096^2 in FP32: forward 0.57 ms (image step 0.24 and cuFFT 1.01), adjoint
+// 0.56 ms (cuFFT 1.03 and image step 0.11), and no library workspace (1 GiB).
+// Bound: the exchanges (the row passes keep the shared-memory pipe 70-78%
+// busy, the column passes 50-57% with 16 warps per SM); DRAM at 4.1-4.3 TB/s
+// in the column passes.  Tried for them: tiles by cp.async into two buffers
+// (0.54 and 0.60 ms), by plain loads and stores 4 columns wide (0.53), 2
+// columns (0.73), 64 registers (0.83, spills).
 //
 // An N-point transform runs over N / 16 threads of 16 values each, in radix-16
 // Stockham steps and a last one of radix N / 16^k, exchanged through shared
@@ -255,9 +256,9 @@ __device__ __forceinline__ void fft_points(C (&v)[16], C* sh, int j, const C* __
 
 // Shared memory of one transform; rows per block of the row passes (a warp
 // at least, and no more than that: small images have few rows); columns
-// per block of the column passes (32 bytes of a row at N = 2048, 128 at most:
-// neighbouring blocks share their lines in L2), each with 16 / C values more,
-// so that the columns of a half-warp meet no bank twice.
+// per tile of the column passes (32 bytes of a row at N = 2048, 128 at most),
+// each column's exchange memory with 16 / C values more, so that the columns
+// of a half-warp meet no bank twice.
 template <int kLog> __host__ __device__ constexpr int fft_row_elems() { return fft_pad(1 << kLog); }
 template <int kLog> __host__ __device__ constexpr int fft_rows() { return kLog >= 9 ? 1 : 1 << (9 - kLog); }
 template <int kLog, typename T> __host__ __device__ constexpr int fft_cols() {
@@ -319,63 +320,228 @@ __global__ void __launch_bounds__(fft_row_threads<kLog>(), (sizeof(T) == 4 ? 512
   }
 }
 
-// Column pass of the forward transform, in place: rows 0 .. N - 1 (image rows)
-// to rows 0 .. 2 N - 1 of the transform.
+// The column passes move their tiles (fft_cols columns of one grid) by TMA:
+// N rows of a tile at a time into shared memory, [row][column], and results
+// out of it, while the tile before is transformed.  A tile's rows are 32 to
+// 128 bytes long and a grid row apart, so that loads and stores by the
+// threads cost the shared-memory pipe one wavefront for each row of a warp's
+// request: 0.53 ms for 8 grids of 4096^2, more than half of it that, against
+// 0.38 (forward) and 0.37 (adjoint).  One block per SM, tiles in turn.
+//
+// The tensor maps (fft_maps): `image` the rows 0 .. N - 1 of every grid,
+// [grid][row][column]; `half` all 2 N rows, [grid][row mod 2][row / 2][column].
+// Boxes of fft_cols columns and min(N, 256) rows.
+__device__ __forceinline__ unsigned fft_smem_addr(const void* p) {
+  return static_cast<unsigned>(__cvta_generic_to_shared(p));
+}
+// TMA boxes start on 128-byte boundaries of shared memory.
+__device__ __forceinline__ unsigned char* fft_aligned(unsigned char* p) {
+  return p + ((128u - fft_smem_addr(p)) & 127u);
+}
+__device__ __forceinline__ void fft_bar_init(unsigned long long* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(fft_smem_addr(bar)) : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+__device__ __forceinline__ void fft_bar_expect(unsigned long long* bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fft_smem_addr(bar)),
+               "r"(bytes)
+               : "memory");
+}
+// Waits for the phase of the given parity, for at most about a second; false
+// if it did not complete (the block then records it and leaves).
+__device__ __forceinline__ bool fft_bar_wait(unsigned long long* bar, unsigned parity) {
+  for (int i = 0; i < (1 << 20); ++i) {
+    unsigned done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(fft_smem_addr(bar)), "r"(parity)
+        : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+// N rows of a tile into buf: rows of the image map, or rows of one parity of
+// the half map (one thread).
+template <typename C, int N, int NC, bool kHalf>
+__device__ __forceinline__ void fft_tile_load(C* buf, const FftMaps* maps, int col, int parity,
+                                              int grid, unsigned long long* bar) {
+  constexpr int kBox = N < 256 ? N : 256;
+  fft_bar_expect(bar, static_cast<unsigned>(sizeof(C)) * N * NC);
+  // columns in 8-byte units
+  const int x = col * static_cast<int>(sizeof(C) / 8);
+#pragma unroll 1
+  for (int r = 0; r < N; r += kBox) {
+    const unsigned dst = fft_smem_addr(buf + r * NC);
+    if (kHalf)
+      asm volatile(
+          "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], "
+          "[%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+          "l"(&maps->half), "r"(x), "r"(r), "r"(parity), "r"(grid), "r"(fft_smem_addr(bar))
+          : "memory");
+    else
+      asm volatile(
+          "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], "
+          "[%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+          "l"(&maps->image), "r"(x), "r"(r), "r"(grid), "r"(fft_smem_addr(bar))
+          : "memory");
+  }
+}
+// The same rows from buf to the grid (one thread, after fft_publish).
+template <typename C, int N, int NC, bool kHalf>
+__device__ __forceinline__ void fft_tile_store(const C* buf, const FftMaps* maps, int col,
+                                               int parity, int grid) {
+  constexpr int kBox = N < 256 ? N : 256;
+  const int x = col * static_cast<int>(sizeof(C) / 8);
+#pragma unroll 1
+  for (int r = 0; r < N; r += kBox) {
+    const unsigned src = fft_smem_addr(buf + r * NC);
+    if (kHalf)
+      asm volatile(
+          "cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];" ::"l"(
+              &maps->half),
+          "r"(x), "r"(r), "r"(parity), "r"(grid), "r"(src)
+          : "memory");
+    else
+      asm volatile(
+          "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+              &maps->image),
+          "r"(x), "r"(r), "r"(grid), "r"(src)
+          : "memory");
+  }
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void fft_stores_read() {   // their source may be rewritten
+  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+__device__ __forceinline__ void fft_stores_done() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+// Makes this thread's writes to shared memory visible to the TMA unit.
+__device__ __forceinline__ void fft_publish() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Column pass of the forward transform, in place: rows 0 .. N - 1 (image
+// rows) to rows 0 .. 2 N - 1 of the transform, even ones first.
 template <typename T, typename C, int kLog>
-__global__ void __launch_bounds__(fft_col_threads<kLog, T>(),
-                                  (sizeof(T) == 4 ? 512 : 256) / fft_col_threads<kLog, T>())
-    fft_cols_forward_kernel(const C* __restrict__ tab, C* grids) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int N = 1 << kLog, TPC = N / 16, NC = fft_cols<kLog, T>();
+__global__ void __launch_bounds__(fft_col_threads<kLog, T>())
+    fft_cols_forward_kernel(const C* __restrict__ tab, const __grid_constant__ FftMaps maps,
+                            int tiles, int* __restrict__ timeout) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(8) unsigned long long bar;
+  constexpr int N = 1 << kLog, TPC = N / 16, NC = fft_cols<kLog, T>(), kTiles = 2 * N / NC;
   const int c = threadIdx.x % NC, j = threadIdx.x / NC;
-  C* sh = reinterpret_cast<C*>(smem_raw) + c * fft_col_elems<kLog, T>();
-  C* col = grids + static_cast<int64_t>(blockIdx.y) * 4 * N * N + blockIdx.x * NC + c;
-  C in[16], v[16];
-#pragma unroll
-  for (int m = 0; m < 16; ++m) {
-    const int n = j + m * TPC;
-    in[m] = col[static_cast<int64_t>(n ^ (N / 2)) * 2 * N];
-    v[m] = in[m];
+  C* in = reinterpret_cast<C*>(fft_aligned(smem_raw));
+  C* out = in + N * NC;
+  C* sh = out + N * NC + c * fft_col_elems<kLog, T>();
+  const bool lead = threadIdx.x == 0;
+  if (lead) {
+    fft_bar_init(&bar);
+    fft_tile_load<C, N, NC, false>(in, &maps, blockIdx.x % kTiles * NC, 0, blockIdx.x / kTiles, &bar);
   }
-  fft_points<kLog, -1>(v, sh, j, tab);
-  // every row of these columns has been read once the block has passed its
-  // first exchange, which precedes this point for all of its threads
+  __syncthreads();
+  unsigned parity = 0;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, parity ^= 1) {
+    const int col = tile % kTiles * NC, grid = tile / kTiles, next = tile + gridDim.x;
+    if (!fft_bar_wait(&bar, parity)) {
+      if (lead) *timeout = 1;
+      fft_bar_wait(&bar, parity);
+      break;
+    }
+    C v[16];
 #pragma unroll
-  for (int m = 0; m < 16; ++m) col[static_cast<int64_t>(j + m * TPC) * 4 * N] = v[m];
+    for (int m = 0; m < 16; ++m) v[m] = in[((j + m * TPC) ^ (N / 2)) * NC + c];
+    fft_points<kLog, -1>(v, sh, j, tab);
+    if (lead) fft_stores_read();
+    __syncthreads();
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
-    const int n = j + m * TPC;
-    in[m] = fft_mul(in[m], tab[n < N / 2 ? n : n + N]);
+    for (int m = 0; m < 16; ++m) out[(j + m * TPC) * NC + c] = v[m];
+    fft_publish();
+    __syncthreads();
+    if (lead) fft_tile_store<C, N, NC, true>(out, &maps, col, 0, grid);
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      const int n = j + m * TPC;
+      v[m] = fft_mul(in[(n ^ (N / 2)) * NC + c], tab[n < N / 2 ? n : n + N]);
+    }
+    __syncthreads();   // the tile has been read
+    if (lead && next < tiles)
+      fft_tile_load<C, N, NC, false>(in, &maps, next % kTiles * NC, 0, next / kTiles, &bar);
+    fft_points<kLog, -1>(v, sh, j, tab);
+    if (lead) fft_stores_read();
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < 16; ++m) out[(j + m * TPC) * NC + c] = v[m];
+    fft_publish();
+    __syncthreads();
+    if (lead) fft_tile_store<C, N, NC, true>(out, &maps, col, 1, grid);
   }
-  fft_points<kLog, -1>(in, sh, j, tab);
-#pragma unroll
-  for (int m = 0; m < 16; ++m) col[static_cast<int64_t>(j + m * TPC) * 4 * N + 2 * N] = in[m];
+  if (lead) fft_stores_done();
 }
 
-// Column pass of the adjoint, in place: 2 N rows to rows 0 .. N - 1 (image rows).
+// Column pass of the adjoint, in place: 2 N rows to rows 0 .. N - 1 (image
+// rows).  One buffer for the even rows and one for the odd, each refilled as
+// soon as it has been read; the results leave from the exchange's memory (from
+// the even rows' buffer, which then waited for them: 0.52 ms).
 template <typename T, typename C, int kLog>
-__global__ void __launch_bounds__(fft_col_threads<kLog, T>(),
-                                  (sizeof(T) == 4 ? 512 : 256) / fft_col_threads<kLog, T>())
-    fft_cols_adjoint_kernel(const C* __restrict__ tab, C* grids) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int N = 1 << kLog, TPC = N / 16, NC = fft_cols<kLog, T>();
+__global__ void __launch_bounds__(fft_col_threads<kLog, T>())
+    fft_cols_adjoint_kernel(const C* __restrict__ tab, const __grid_constant__ FftMaps maps,
+                            int tiles, int* __restrict__ timeout) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ __align__(8) unsigned long long bars[2];
+  constexpr int N = 1 << kLog, TPC = N / 16, NC = fft_cols<kLog, T>(), kTiles = 2 * N / NC;
   const int c = threadIdx.x % NC, j = threadIdx.x / NC;
-  C* sh = reinterpret_cast<C*>(smem_raw) + c * fft_col_elems<kLog, T>();
-  C* col = grids + static_cast<int64_t>(blockIdx.y) * 4 * N * N + blockIdx.x * NC + c;
-  C even[16], v[16];
-#pragma unroll
-  for (int m = 0; m < 16; ++m) even[m] = col[static_cast<int64_t>(j + m * TPC) * 4 * N];
-#pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = col[static_cast<int64_t>(j + m * TPC) * 4 * N + 2 * N];
-  fft_points<kLog, 1>(even, sh, j, tab);
-  fft_points<kLog, 1>(v, sh, j, tab);
-  // (both sets of rows were read before the first exchange)
-#pragma unroll
-  for (int m = 0; m < 16; ++m) {
-    const int n = j + m * TPC;
-    const C o = fft_add(even[m], fft_mul(v[m], fft_root<1>(tab[n < N / 2 ? n : n + N])));
-    col[static_cast<int64_t>(n ^ (N / 2)) * 2 * N] = o;
+  C* buf = reinterpret_cast<C*>(fft_aligned(smem_raw));   // even rows
+  C* buf1 = buf + N * NC;                                 // odd rows
+  C* out = buf1 + N * NC;                                 // results, over the exchange
+  C* sh = out + c * fft_col_elems<kLog, T>();
+  const bool lead = threadIdx.x == 0;
+  if (lead) {
+    fft_bar_init(&bars[0]);
+    fft_bar_init(&bars[1]);
+    const int col = blockIdx.x % kTiles * NC, grid = blockIdx.x / kTiles;
+    fft_tile_load<C, N, NC, true>(buf, &maps, col, 0, grid, &bars[0]);
+    fft_tile_load<C, N, NC, true>(buf1, &maps, col, 1, grid, &bars[1]);
   }
+  __syncthreads();
+  unsigned parity = 0;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, parity ^= 1) {
+    const int col = tile % kTiles * NC, grid = tile / kTiles, next = tile + gridDim.x;
+    C even[16], v[16];
+    if (!fft_bar_wait(&bars[0], parity)) {
+      if (lead) *timeout = 1;
+      fft_bar_wait(&bars[0], parity);
+      break;
+    }
+#pragma unroll
+    for (int m = 0; m < 16; ++m) even[m] = buf[(j + m * TPC) * NC + c];
+    if (lead) fft_stores_read();   // the exchange's memory is free again
+    __syncthreads();               // and the even rows have been read
+    if (lead && next < tiles)
+      fft_tile_load<C, N, NC, true>(buf, &maps, next % kTiles * NC, 0, next / kTiles, &bars[0]);
+    fft_points<kLog, 1>(even, sh, j, tab);
+    if (!fft_bar_wait(&bars[1], parity)) {
+      if (lead) *timeout = 1;
+      fft_bar_wait(&bars[1], parity);
+      break;
+    }
+#pragma unroll
+    for (int m = 0; m < 16; ++m) v[m] = buf1[(j + m * TPC) * NC + c];
+    __syncthreads();               // the odd rows have been read
+    if (lead && next < tiles)
+      fft_tile_load<C, N, NC, true>(buf1, &maps, next % kTiles * NC, 1, next / kTiles, &bars[1]);
+    fft_points<kLog, 1>(v, sh, j, tab);
+    __syncthreads();               // the last exchange has been read
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      const int n = j + m * TPC;
+      out[(n ^ (N / 2)) * NC + c] =
+          fft_add(even[m], fft_mul(v[m], fft_root<1>(tab[n < N / 2 ? n : n + N])));
+    }
+    fft_publish();
+    __syncthreads();
+    if (lead) fft_tile_store<C, N, NC, false>(out, &maps, col, 0, grid);
+  }
+  if (lead) fft_stores_done();
 }
 
 // Row pass of the adjoint: row p of every grid of the group, times conj(S~_k),

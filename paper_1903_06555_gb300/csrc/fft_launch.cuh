@@ -5,14 +5,67 @@
 
 enum FftPass { kFftRowsForward, kFftColsForward, kFftColsAdjoint, kFftRowsAdjoint };
 
+// Shared memory of a column block: two tile buffers, the exchange, and room
+// to align them.
+template <typename T, typename C, int kLog>
+constexpr size_t fft_col_smem() {
+  return 128 + sizeof(C) * fft_cols<kLog, T>() *
+                   (2 * (size_t(1) << kLog) + fft_col_elems<kLog, T>());
+}
+
+// The tensor maps of the plan's grids (fft_kernel.cuh says what they show).
+template <typename T, typename C, int kLog>
+int fft_make_maps_log(Plan& p) {
+  constexpr uint64_t N = uint64_t(1) << kLog, row = 2 * N * sizeof(C);
+  constexpr uint32_t kBox = N < 256 ? N : 256;
+  constexpr uint32_t unit = sizeof(C) / 8;   // 8-byte elements per grid value
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult found;
+  PHI_CUDA_TRY(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
+                                                cudaEnableDefault, &found));
+  if (found != cudaDriverEntryPointSuccess || !fn) return PHI_ERR_CUDA;
+  typedef CUresult (*Encode)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
+                             const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                             const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  auto encode = [&](CUtensorMap* map, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                    const cuuint32_t* box) {
+    const cuuint32_t one[4] = {1, 1, 1, 1};
+    return reinterpret_cast<Encode>(fn)(
+               map, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, rank, p.grid, dims, strides, box, one,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+               ? PHI_OK
+               : PHI_ERR_CUDA;
+  };
+  const uint64_t grids = static_cast<uint64_t>(p.group);
+  const cuuint64_t idims[3] = {2 * N * unit, N, grids}, istr[2] = {row, 2 * N * row};
+  const cuuint32_t ibox[3] = {fft_cols<kLog, T>() * unit, kBox, 1};
+  PHI_TRY_ST(encode(&p.fft_maps.image, 3, idims, istr, ibox));
+  const cuuint64_t hdims[4] = {2 * N * unit, N, 2, grids};
+  const cuuint64_t hstr[3] = {2 * row, row, 2 * N * row};
+  const cuuint32_t hbox[4] = {fft_cols<kLog, T>() * unit, kBox, 1, 1};
+  return encode(&p.fft_maps.half, 4, hdims, hstr, hbox);
+}
+
 template <typename T, typename C, int kLog>
 int fft_pass_log(Plan& p, FftPass pass, const int32_t* stacks, int n, const T* x_in, C* grids,
                  T* x_out, int accumulate, cudaStream_t s) {
   constexpr int N = 1 << kLog;
   constexpr int row_threads = fft_row_threads<kLog>(), col_threads = fft_col_threads<kLog, T>();
   constexpr size_t row_smem = sizeof(C) * fft_rows<kLog>() * fft_row_elems<kLog>();
-  constexpr size_t col_smem = sizeof(C) * fft_cols<kLog, T>() * fft_col_elems<kLog, T>();
-  const dim3 rows(n, N / fft_rows<kLog>()), cols(2 * N / fft_cols<kLog, T>(), n);
+  constexpr size_t col_smem = fft_col_smem<T, C, kLog>();
+  const dim3 rows(n, N / fft_rows<kLog>());
+  const int tiles = 2 * N / fft_cols<kLog, T>() * n;
+  int* timeout = reinterpret_cast<int*>(p.counters + p.K + 4);
+  auto cols = [&](auto kernel) {   // as many blocks as run at once, and no more than tiles
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, col_threads, col_smem) !=
+            cudaSuccess ||
+        per_sm < 1)
+      per_sm = 1;
+    return std::min(tiles, per_sm * p.num_sms);
+  };
   const auto* omn = static_cast<const typename PixelPhase<T>::omn*>(p.omn_pix);
   const T* corr = static_cast<const T*>(p.corr_pix);
   const C* tab = static_cast<const C*>(p.fft_tab);
@@ -22,10 +75,14 @@ int fft_pass_log(Plan& p, FftPass pass, const int32_t* stacks, int n, const T* x
           x_in, omn, corr, p.wbar_dev, stacks, tab, grids);
       break;
     case kFftColsForward:
-      fft_cols_forward_kernel<T, C, kLog><<<cols, col_threads, col_smem, s>>>(tab, grids);
+      fft_cols_forward_kernel<T, C, kLog>
+          <<<cols(fft_cols_forward_kernel<T, C, kLog>), col_threads, col_smem, s>>>(
+              tab, p.fft_maps, tiles, timeout);
       break;
     case kFftColsAdjoint:
-      fft_cols_adjoint_kernel<T, C, kLog><<<cols, col_threads, col_smem, s>>>(tab, grids);
+      fft_cols_adjoint_kernel<T, C, kLog>
+          <<<cols(fft_cols_adjoint_kernel<T, C, kLog>), col_threads, col_smem, s>>>(
+              tab, p.fft_maps, tiles, timeout);
       break;
     case kFftRowsAdjoint:
       fft_rows_adjoint_kernel<T, C, kLog><<<rows.y, row_threads, row_smem, s>>>(
@@ -49,25 +106,27 @@ int fft_pass(Plan& p, FftPass pass, const int32_t* stacks, int n, const T* x_in,
   }
 }
 
-// Dynamic shared memory limits (fixed per kernel, the same for every plan).
+// Dynamic shared memory limits (fixed per kernel, the same for every plan) and
+// the plan's tensor maps.
 template <typename T, typename C, int kLog>
-int set_fft_smem_log() {
+int fft_setup_log(Plan& p) {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   const int row = static_cast<int>(sizeof(C) * fft_rows<kLog>() * fft_row_elems<kLog>());
-  const int col = static_cast<int>(sizeof(C) * fft_cols<kLog, T>() * fft_col_elems<kLog, T>());
+  const int col = static_cast<int>(fft_col_smem<T, C, kLog>());
   PHI_CUDA_TRY(cudaFuncSetAttribute(fft_rows_forward_kernel<T, C, kLog>, a, row));
   PHI_CUDA_TRY(cudaFuncSetAttribute(fft_rows_adjoint_kernel<T, C, kLog>, a, row));
   PHI_CUDA_TRY(cudaFuncSetAttribute(fft_cols_forward_kernel<T, C, kLog>, a, col));
   PHI_CUDA_TRY(cudaFuncSetAttribute(fft_cols_adjoint_kernel<T, C, kLog>, a, col));
-  return PHI_OK;
+  return fft_make_maps_log<T, C, kLog>(p);
 }
 template <typename T, typename C>
-int set_fft_smem() {
-  PHI_TRY_ST((set_fft_smem_log<T, C, 6>()));
-  PHI_TRY_ST((set_fft_smem_log<T, C, 7>()));
-  PHI_TRY_ST((set_fft_smem_log<T, C, 8>()));
-  PHI_TRY_ST((set_fft_smem_log<T, C, 9>()));
-  PHI_TRY_ST((set_fft_smem_log<T, C, 10>()));
-  PHI_TRY_ST((set_fft_smem_log<T, C, 11>()));
-  return PHI_OK;
+int fft_setup(Plan& p) {
+  switch (p.fft_log) {
+    case 6: return fft_setup_log<T, C, 6>(p);
+    case 7: return fft_setup_log<T, C, 7>(p);
+    case 8: return fft_setup_log<T, C, 8>(p);
+    case 9: return fft_setup_log<T, C, 9>(p);
+    case 10: return fft_setup_log<T, C, 10>(p);
+    default: return fft_setup_log<T, C, 11>(p);
+  }
 }

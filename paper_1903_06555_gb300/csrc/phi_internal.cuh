@@ -24,6 +24,7 @@
 //                       are rounded into the complex grids.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <cufft.h>
 #include <stdint.h>
@@ -161,6 +162,11 @@ struct QuadParams {
   FixedGrid fx;               // gridding target of deterministic plans
 };
 
+// Tensor maps of the resident grids, for the two-pass transforms' columns.
+struct FftMaps {
+  CUtensorMap image, half;
+};
+
 struct Plan {
   phi_plan_desc d;
   int N = 0, npad = 0, K = 0;
@@ -194,9 +200,11 @@ struct Plan {
   int fft_batch_n = 1;
   int fft_log = 0;                      // two-pass transforms: log2 N (0: cuFFT)
   void* fft_tab = nullptr;              // their roots of unity
+  FftMaps fft_maps;
   bool fft_batch_ok = false;
   // [0..K) work heads, [K] unconverged taps, [K+1] taps, [K+2] wkernel misses,
-  // [K+3] tap-node evaluations; retry_counters[2 g], [2 g + 1], g < K: length
+  // [K+3] node evaluations, [K+4] a transform's bounded wait ran out;
+  // retry_counters[2 g], [2 g + 1], g < K: length
   // of group g's retry list and the head of the queue that takes it, just
   // before the work heads so that one memset clears both
   unsigned long long* counters = nullptr;

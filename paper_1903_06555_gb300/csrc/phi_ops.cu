@@ -2342,6 +2342,10 @@ int fft_two_pass_log(int N, int npad, bool f64) { return fft_log(N, npad, f64); 
 int fft_two_pass_table(int N) { return fft_table_size(N); }
 
 int build_fft_table(Plan& p, cudaStream_t s) {
+  if (p.d.precision == PHI_F64)
+    PHI_TRY_ST((fft_setup<double, double2>(p)));
+  else
+    PHI_TRY_ST((fft_setup<float, float2>(p)));
   const int blocks = (fft_table_size(p.N) + 255) / 256;
   if (p.d.precision == PHI_F64)
     fft_table_kernel<double, double2><<<blocks, 256, 0, s>>>(p.fft_log,
@@ -2471,8 +2475,6 @@ int set_kernel_smem_limits() {
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
   PHI_CUDA_TRY(cudaFuncSetAttribute(vis_radial_kernel<double, double2, true>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-  PHI_TRY_ST((set_fft_smem<float, float2>()));
-  PHI_TRY_ST((set_fft_smem<double, double2>()));
   PHI_CUDA_TRY((set_series_smem<float, float2>(optin)));
   PHI_CUDA_TRY((set_series_smem<double, double2>(optin)));
   PHI_CUDA_TRY((set_dde_smem<float, float2>(optin)));

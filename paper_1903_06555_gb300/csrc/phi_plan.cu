@@ -481,9 +481,9 @@ int build(Plan& p, const double* uvw, const double* weights, int64_t M, cudaStre
   p.stack_off.assign(K + 1, 0);
   p.stack_jw.assign(K, 0);
   p.stack_maxabs.assign(K, 0.0);
-  PHI_CUDA_TRY(owned_alloc(p, &p.retry_counters, 3 * static_cast<size_t>(K) + 4));
+  PHI_CUDA_TRY(owned_alloc(p, &p.retry_counters, 3 * static_cast<size_t>(K) + 5));
   p.counters = p.retry_counters + 2 * K;
-  PHI_CUDA_TRY(cudaMemsetAsync(p.retry_counters, 0, sizeof(unsigned long long) * (3 * K + 4), s));
+  PHI_CUDA_TRY(cudaMemsetAsync(p.retry_counters, 0, sizeof(unsigned long long) * (3 * K + 5), s));
 
   Scratch tmp;
   const int nblk = std::max(1, std::min<int>(p.num_sms * 4,
@@ -980,17 +980,17 @@ extern "C" int phi_plan_stats(phi_plan_t plan, int64_t* n_unconverged, int64_t* 
                               int64_t* n_tap_nodes, int reset, void* stream) {
   if (!plan) return PHI_ERR_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  unsigned long long h[4] = {0, 0, 0, 0};
+  unsigned long long h[5] = {0, 0, 0, 0, 0};
   PHI_CUDA_TRY(cudaMemcpyAsync(h, plan->counters + plan->K, sizeof(h), cudaMemcpyDeviceToHost, s));
   PHI_CUDA_TRY(cudaStreamSynchronize(s));
   if (n_unconverged) *n_unconverged = static_cast<int64_t>(h[0]);
   if (n_taps) *n_taps = static_cast<int64_t>(h[1]);
   if (n_tap_nodes) *n_tap_nodes = static_cast<int64_t>(h[3]);
   if (reset) {
-    PHI_CUDA_TRY(cudaMemsetAsync(plan->counters + plan->K, 0, 4 * sizeof(unsigned long long), s));
+    PHI_CUDA_TRY(cudaMemsetAsync(plan->counters + plan->K, 0, sizeof(h), s));
     PHI_CUDA_TRY(cudaStreamSynchronize(s));
   }
-  return PHI_OK;
+  return h[4] ? PHI_ERR_TIMEOUT : PHI_OK;
 }
 
 extern "C" const char* phi_error_string(int status) {

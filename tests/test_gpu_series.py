@@ -41,7 +41,7 @@ def observation(geo, jw, n, seed):
                          + [("f64", j) for j in (4, 8, 10, 30, 32, 52, 54, 74, 76, 90)])
 def test_supports_match_oracle(precision, jw):
     geo = O.Geometry(64, 2.0, math.radians(20.0), 4.0, tol_rel=1e-13, tol_abs=1e-13)
-    n = 24 if jw > 50 else 120
+    n = 12 if jw > 50 else 60
     uvw = observation(geo, jw, n, jw)
     op = O.make_plan(uvw, geo, 1, False, max_support=128)
     assert op.jw.max() == jw
