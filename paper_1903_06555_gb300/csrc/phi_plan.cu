@@ -685,7 +685,12 @@ int build(Plan& p, const double* uvw, const double* weights, int64_t M, cudaStre
     if (p.stack_off[q + 1] > p.stack_off[q]) p.group_stacks.push_back(q);
   const double budget = (d.max_grid_mib > 0 ? d.max_grid_mib : 4096) * 1048576.0;
   p.group = static_cast<int>(std::max<double>(1.0, std::floor(budget / (grid_bytes + fx_bytes))));
-  p.group = std::max(1, std::min<int>(p.group, static_cast<int>(p.group_stacks.size())));
+  const int shown = std::max(1, static_cast<int>(p.group_stacks.size()));
+  p.group = std::max(1, std::min(p.group, shown));
+  // groups of equal size, no more of them: less memory to set up and give back
+  // (50 stacks of 4096^2 in 4 GiB: 25 + 25 in place of 32 + 18, 0.9 GB less)
+  const int ngroups = (shown + p.group - 1) / p.group;
+  p.group = (shown + ngroups - 1) / ngroups;
   p.group_off.assign(1, 0);
   for (size_t g = 0; g < p.group_stacks.size(); g += p.group)
     p.group_off.push_back(static_cast<int64_t>(std::min(p.group_stacks.size(), g + p.group)));
