@@ -37,11 +37,9 @@ import workloads as W  # noqa: E402
 
 METRIC = "w-corrected visibilities/s (degrid+grid) at <=1e-5 rel err vs FP64; p50/p99 latency"
 UNIT = "vis/s"
-FLOPS_PER_TAP_NODE = 36.0     # J0 by a rational/asymptotic approximation (28) + 2 weighted complex MACs (8)
+FLOPS_PER_TAP_NODE = 36.0     # the oracle's work: J0 by a rational/asymptotic approximation (28) + 2 weighted complex MACs (8)
 FP32_LANES_PER_SM = 128       # FP32 FMA lanes per SM per clock (Blackwell)
 FP64_NOMINAL_TFLOPS = 1.25   # GB300 dense FP64, nominal
-RADIAL_POINTS = 16            # Chebyshev points per piece, FP32 radial mode
-RADIAL_FLOPS_PER_TAP = 96     # 15 Clenshaw steps x (2 FMA + 2 subtractions) + the last step
 
 
 def parse():
@@ -222,7 +220,7 @@ def kernel_source_hash():
     import hashlib
     h = hashlib.sha256()
     for f in ("phi_ops.cu", "bessel_j0.cuh", "phi_internal.cuh", "table_index.cuh",
-              "fixed_point.cuh"):
+              "fixed_point.cuh", "series_kernel.cuh", "series_coef.cuh", "fft_kernel.cuh"):
         with open(os.path.join(ROOT, "paper_1903_06555_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -231,7 +229,7 @@ def kernel_source_hash():
 def profiled_traffic(stage):
     """DRAM bytes per launch of the fused kernel from the committed ncu launch
     list, or None when the kernel sources changed since it was taken."""
-    p = os.path.join(ROOT, "profiles", "vis_kernel_mwa-2048-8stack_launches.md")
+    p = os.path.join(ROOT, "profiles", "vis_series_kernel_mwa-2048.md")
     if not os.path.exists(p):
         return None
     vals = {}
@@ -247,30 +245,10 @@ def profiled_traffic(stage):
 
 
 def profiled_pipes():
-    """FMA-pipe and issue-slot activity of the fused degrid kernel from the
-    committed small-case ncu capture, or None when the kernel sources changed
-    since it was taken."""
-    p = os.path.join(ROOT, "profiles", "vis_kernel_degrid_mwa-2048-first40000_full.md")
-    if not os.path.exists(p):
-        return None
-    vals = {}
-    for line in open(p):
-        if ":" in line:
-            k, v = line.split(":", 1)
-            vals[k.strip()] = v.strip()
-    if vals.get("kernel_source_sha256") != kernel_source_hash():
-        return None
-    keys = ("fma_pipe_pct", "fma_heavy_pipe_pct", "issue_active_pct", "warp_inst_per_tap_node")
-    out = {k: float(vals[k]) for k in keys if k in vals}
-    out["source"] = "profiles/vis_kernel_degrid_mwa-2048-first40000_full.md (40,000-visibility case)"
-    return out
-
-
-def profiled_fp64():
-    """DP flops per tap-node and FP64-pipe activity of vis_kernel<double> from
-    the committed small-case ncu capture, or None when the kernel sources
+    """Shared-memory pipe, issue and FMA activity of the fused degrid kernel
+    from the committed small-case ncu capture, or None when the kernel sources
     changed since it was taken."""
-    p = os.path.join(ROOT, "profiles", "vis_kernel_f64_degrid_mwa-2048-first2000.md")
+    p = os.path.join(ROOT, "profiles", "vis_series_kernel_mwa-2048.md")
     if not os.path.exists(p):
         return None
     vals = {}
@@ -280,10 +258,30 @@ def profiled_fp64():
             vals[k.strip()] = v.strip()
     if vals.get("kernel_source_sha256") != kernel_source_hash():
         return None
-    keys = ("fp64_flops_per_tap_node", "fp64_pipe_pct", "issue_active_pct")
+    keys = ("lsu_wavefront_pct", "issue_active_pct", "fma_pipe_pct", "warp_inst_per_vis")
     out = {k: float(vals[k]) for k in keys if k in vals}
-    out["source"] = "profiles/vis_kernel_f64_degrid_mwa-2048-first2000.md"
+    out["source"] = "profiles/vis_series_kernel_mwa-2048.md (200,007-visibility case)"
     return out
+
+
+def series_intervals(info):
+    """Sample intervals summed over the kept visibilities of one call (the
+    library's series_intervals over each stack's support)."""
+    inv = 4.0 * info["window_radius"]
+    return sum(c * (int(j * 0.70710678 * inv + 1e-3) + 1)
+               for c, j in zip(info["counts"], info["jw"]) if j)
+
+
+def series_flops(sample_nodes, intervals, taps, f64=False):
+    """Flops of the sampled quadrature, degrid or grid: per sample and node the
+    Kronrod sum (a real times a complex multiply-add, 4) and at 15 of 31 nodes
+    the Gauss sum; per sample interval 10 (FP64: 20) sample pairs, each added
+    and subtracted and accumulated in 8 (14) polynomial terms; per tap the
+    polynomial (4 flops a term but the first), its distance (10; FP64 about
+    30 with the square root) and its application (8)."""
+    pairs, terms, dist = (20, 14, 30) if f64 else (10, 8, 10)
+    return (sample_nodes * 4.0 * (1.0 + 15.0 / 31.0) + intervals * pairs * (4.0 + 4.0 * terms) +
+            taps * (4.0 * (terms - 1) + dist + 8.0))
 
 
 def load_oracle_counts():
@@ -521,9 +519,7 @@ def run_ours(args, ws, rank, local):
                           "bytes": 16 * info["table_n_rho"] * (info["table_n_w"] - 1),
                           "rel_l2_vs_quadrature_path": rel_q}
         else:
-            radial_info = {"piece_width_px": 2.0 / info["window_radius"],
-                           "points_per_piece": RADIAL_POINTS,
-                           "quadrature_points_per_vis": tap_nodes / (2 * args.steps * n_kept),
+            radial_info = {"quadrature_points_per_vis": tap_nodes / (2 * args.steps * n_kept),
                            "rel_l2_vs_quadrature_path": rel_q}
 
     # deterministic gridding beside the default: the same phi_grid call on a
@@ -590,62 +586,51 @@ def run_ours(args, ws, rank, local):
                              "8 B per grid cell covered by a kernel box, the plane pairs once "
                              "per launch; the kernel is bound by its shared-memory reads (L1/TEX "
                              "86-94% busy in ncu for the w-row kernel), far below the HBM roofline"}
-    elif args.kernel_mode == "radial":
-        # executed work: the quadrature at the Chebyshev points (tap-nodes) and
-        # the series evaluated at every tap; degrid and grid do the same work
-        per_launch = (tap_nodes * FLOPS_PER_TAP_NODE + taps * RADIAL_FLOPS_PER_TAP) / (2.0 * n_dom)
-        ach = per_launch / ((ms_dom / n_dom) / 1e3) / 1e12
-        roof = {"bound": "alu", "kernel": f"vis_radial_kernel ({dom})", "achieved": ach,
-                "peak": peak_fp32, "unit": "TFLOP/s", "frac": ach / peak_fp32,
-                "traffic": profiled_traffic("radial_" + dom),
-                "peak_note": f"FP32 FMA: {sms} SMs (device count) x {FP32_LANES_PER_SM} lanes x 2 flops x "
-                             f"{sm_mhz:.0f} MHz (recipe unit counts, max clock)",
-                "work_note": f"{FLOPS_PER_TAP_NODE:.0f} flops per quadrature tap-node at the "
-                             f"Chebyshev points + {RADIAL_FLOPS_PER_TAP} flops per tap for its "
-                             "series (executed work, not the oracle's per-tap count)"}
-    elif f64:
-        # FP64 path: DP flops per tap-node from the committed ncu capture of
-        # vis_kernel<double> (its DFMA/DMUL/DADD counts over the tap-nodes of
-        # the captured launch) x this run's tap-nodes, against the FP64 peak
-        gpu_nodes = tap_nodes / (2 * args.steps * n_kept)
-        prof = profiled_fp64()
-        peak64 = FP64_NOMINAL_TFLOPS * sms / 152.0 * sm_mhz / 2070.0
-        ach = None
-        if prof and "fp64_flops_per_tap_node" in prof:
-            ach = n_kept * gpu_nodes * prof["fp64_flops_per_tap_node"] / launches_per_step / \
-                ((ms_dom / n_dom) / 1e3) / 1e12
-        roof = {"bound": "fp64", "kernel": f"vis_kernel<double> ({dom})", "achieved": ach,
-                "peak": peak64, "unit": "TFLOP/s", "frac": ach / peak64 if ach else None,
-                "traffic": None, "ncu": prof,
-                "peak_note": f"nominal FP64 {FP64_NOMINAL_TFLOPS} TFLOP/s at 152 SMs, 2070 MHz, "
-                             f"scaled to {sms} SMs and {sm_mhz:.0f} MHz (no measured FP64 peak)",
-                "work_note": f"{gpu_nodes:.0f} tap-nodes per visibility (GK 15/31 at tol 1e-12) "
-                             "x the DP flops per tap-node counted by ncu"}
     else:
-        # executed work: the tap-nodes this run's launches evaluated (counted
-        # on the device, refinements included) x the flops of one tap-node
-        gpu_nodes = tap_nodes / (2 * args.steps * n_kept)
-        ex = n_kept * gpu_nodes * FLOPS_PER_TAP_NODE / launches_per_step / \
-            ((ms_dom / n_dom) / 1e3) / 1e12
-        roof = {"bound": "alu", "kernel": f"vis_kernel ({dom})", "achieved": ex,
-                "peak": peak_fp32, "unit": "TFLOP/s", "frac": ex / peak_fp32,
-                "traffic": profiled_traffic(dom),
-                "peak_note": f"FP32 FMA: {sms} SMs (device count) x {FP32_LANES_PER_SM} lanes x 2 flops x "
-                             f"{sm_mhz:.0f} MHz (recipe unit counts, max clock)",
-                "work_note": f"{FLOPS_PER_TAP_NODE:.0f} flops per tap-node x the tap-nodes the "
-                             f"launch evaluated ({gpu_nodes:.0f} per visibility, Gauss-Kronrod "
-                             "15/31 on shared equal panels, refinements included)",
-                # the same flops over the oracle's own count (globally adaptive
-                # GK 7/15 per tap at tol 1e-6): credits the quadrature schedule
-                # as well as the kernel, so it can exceed the peak
-                "oracle_work": {"tap_nodes_per_vis": evals_per_vis, "achieved": achieved,
-                                "frac": achieved / peak_fp32}}
-        roof["ncu"] = profiled_pipes()
+        # the sampled quadrature (quadrature and radial mode): FP32 against the
+        # shared-memory pipe, whose 128 bytes per clock and SM carry 64 bytes of
+        # polynomial and the grid cell of every tap; FP64 against the FP64 pipe
+        calls = 2.0 * args.steps
+        nodes, tp, iv = tap_nodes / calls, taps / calls, series_intervals(info)
+        secs = launches_per_step * (ms_dom / n_dom) / 1e3
+        flops = series_flops(nodes, iv, tp, f64)
+        work_note = (f"{nodes / n_kept:.0f} (sample, node) products, {iv / n_kept:.0f} sample "
+                     f"intervals and {tp / n_kept:.0f} taps per visibility (Gauss-Kronrod 15/31 "
+                     "panel sums at samples in rho, every tap interpolated)")
+        if f64:
+            peak64 = FP64_NOMINAL_TFLOPS * sms / 152.0 * sm_mhz / 2070.0
+            roof = {"bound": "fp64", "kernel": f"vis_series_kernel<double> ({dom})",
+                    "achieved": flops / secs / 1e12, "peak": peak64, "unit": "TFLOP/s",
+                    "frac": flops / secs / 1e12 / peak64, "traffic": None,
+                    "peak_note": f"nominal FP64 {FP64_NOMINAL_TFLOPS} TFLOP/s at 152 SMs, 2070 MHz, "
+                                 f"scaled to {sms} SMs and {sm_mhz:.0f} MHz (no measured FP64 peak)",
+                    "work_note": work_note}
+        else:
+            peak_smem = sms * 128.0 * sm_mhz * 1e6 / 1e12
+            ach = tp * (64.0 + 8.0) / secs / 1e12
+            roof = {"bound": "smem", "kernel": f"vis_series_kernel ({dom})", "achieved": ach,
+                    "peak": peak_smem, "unit": "TB/s", "frac": ach / peak_smem,
+                    "traffic": profiled_traffic(dom),
+                    "peak_note": f"L1/shared data pipe: {sms} SMs (device count) x 128 B x "
+                                 f"{sm_mhz:.0f} MHz",
+                    "work_note": work_note + "; 64 B of polynomial and an 8 B grid cell per tap",
+                    "alu": {"achieved": flops / secs / 1e12, "peak": peak_fp32, "unit": "TFLOP/s",
+                            "frac": flops / secs / 1e12 / peak_fp32},
+                    # the oracle's own tap-nodes (globally adaptive GK 7/15 per tap
+                    # at tol 1e-6) over the same time: credits the sharing of the
+                    # node sums between taps, so it exceeds the peak
+                    "oracle_work": {"tap_nodes_per_vis": evals_per_vis, "achieved": achieved,
+                                    "frac": achieved / peak_fp32}}
+            roof["ncu"] = profiled_pipes()
     if roof["traffic"]:
         # HBM moved per launch (committed ncu figure) over this run's launch time
         gbs = roof["traffic"] / ((ms_dom / n_dom) / 1e3) / 1e9
         hbm_peak = peaks.get("hbm_gbs", 6800.0)
         roof["hbm"] = {"achieved_gbs": gbs, "peak_gbs": hbm_peak, "frac": gbs / hbm_peak}
+
+    # grids the library transforms by its own two-pass kernels
+    own_fft = info["npad"] == 2 * wl.image_n and wl.image_n in [2 ** k for k in
+                                                                range(9 if f64 else 6, 12)]
 
     # end to end through the public API from pinned host buffers
     e2e = run_e2e(phi, desc, uvw_np, x_np, args.e2e_steps, dev) if args.e2e_steps > 0 else None
@@ -690,11 +675,16 @@ def run_ours(args, ws, rank, local):
         "deterministic_grid": det_info,
         "e2e": e2e,
         "serving": serving,
-        # this library's kernels in the timed steps (prep, fused degrid, fused
-        # grid, finish: one each per stack group; with deterministic gridding
-        # also the term bound, the exponent and the fixed-point conversion of
-        # each grid launch); cuFFT's and the memsets are not counted
-        "gpu_launches": int(sum(stages[k][1] for k in ("prep", "degrid", "grid", "finish")) +
+        # this library's kernels in the timed steps: the image-domain steps and
+        # the FFT's column pass (cuFFT's kernels are not counted), the fused
+        # degrid and grid and, outside the table mode, the launch over what
+        # they left; with deterministic gridding also the term bound, the
+        # exponent and the fixed-point conversion of each grid launch; the
+        # memsets are not counted
+        "gpu_launches": int(sum(stages[k][1] for k in ("prep", "finish") +
+                                (("fft",) if own_fft else ())) +
+                            sum(stages[k][1] for k in ("degrid", "grid")) *
+                            (1 if args.kernel_mode == "table" else 2) +
                             (3 * stages["grid"][1] if args.grid_deterministic else 0)),
         "clocks": clocks,
         "wall_s_timed": wall,
@@ -1027,22 +1017,20 @@ def run_precision(args):
         return float(torch.linalg.vector_norm(a.to(b.dtype) - b) / torch.linalg.vector_norm(b))
     y64 = p64.degrid(x64)
     g64 = p64.grid(ys.to(torch.complex128))
-    # the FP64 path against the FP64 pipe: DP flops per tap-node from the
-    # committed ncu capture of vis_kernel<double> x the tap-nodes counted here
+    # the FP64 path against the FP64 pipe
     p64.stats_full(reset=True)
     p64.degrid(x64)
     p64.grid(ys.to(torch.complex128))
-    nodes64 = p64.stats_full(reset=True)[2]
-    prof64 = profiled_fp64()
+    _, taps64, nodes64 = p64.stats_full(reset=True)
     peaks = measured_peaks()
     peak64 = FP64_NOMINAL_TFLOPS * device_sms() / 152.0 * peaks.get("sm_max_mhz", 2070.0) / 2070.0
-    fp64_roof = {"tap_nodes_per_vis": nodes64 / (2 * n_sub), "peak": peak64, "unit": "TFLOP/s",
-                 "peak_note": "nominal FP64 (no measured FP64 peak)", "ncu": prof64}
-    if prof64 and "fp64_flops_per_tap_node" in prof64:
-        ach = nodes64 * prof64["fp64_flops_per_tap_node"] / (ms_sub64 / 1e3) / 1e12
-        fp64_roof.update(achieved=ach, frac=ach / peak64,
-                         note="degrid + grid of the sub-observation, FFTs and prep included in "
-                              "the time, so the kernel's own fraction is higher")
+    ach = series_flops(nodes64, 2 * series_intervals(p64.info()), taps64, True) / \
+        (ms_sub64 / 1e3) / 1e12
+    fp64_roof = {"sample_nodes_per_vis": nodes64 / (2 * n_sub), "achieved": ach, "peak": peak64,
+                 "frac": ach / peak64, "unit": "TFLOP/s",
+                 "peak_note": "nominal FP64 (no measured FP64 peak)",
+                 "note": "degrid + grid of the sub-observation, FFTs and prep included in the "
+                         "time, so the kernel's own fraction is higher"}
     # the radial interpolation mode: FP32 at full size, FP32 and FP64 on the
     # sub-observation, both against the FP64 per-tap quadrature
     rplan = phi.Plan(torch.from_numpy(uvw).to(dev), kernel_mode="radial", **kw)
@@ -1185,13 +1173,13 @@ def run_dde(args):
               "rel_l2_vs_quadrature_box": float(torch.linalg.vector_norm(yr - yq) /
                                                 torch.linalg.vector_norm(yq))}
     rplan.close()
-    # executed work: the quadrature tap-nodes of the w-kernel boxes and the
-    # separable convolution's complex multiply-adds (8 flops each): per
-    # visibility of support J_w, J_D J_w^2 for the row pass (J_w rows of the
-    # J_w + J_D - 1 columns, J_D taps inside the box per w-kernel tap) and
-    # J_D J_w (J_w + J_D - 1) for the column pass
+    # work of one call: the sampled quadrature's sums and polynomials, every
+    # w-kernel tap from its polynomial, and the separable convolution's complex
+    # multiply-adds (8 flops each): per visibility of support J_w, J_D J_w^2
+    # for the row pass and J_D J_w (J_w + J_D - 1) for the column pass
     macs = dde_macs(info["counts"], info["jw"], jd)
-    flops = nodes * FLOPS_PER_TAP_NODE / calls + macs * 8.0
+    wtaps = sum(c * j * j for c, j in zip(info["counts"], info["jw"]))
+    flops = series_flops(nodes / calls, series_intervals(info), wtaps) + macs * 8.0
     ach = flops / (ms_dde / 2 / 1e3) / 1e12
     peaks = measured_peaks()
     peak_fp32 = fp32_peak_tflops(device_sms(), peaks.get("sm_max_mhz", 2070.0))
@@ -1204,11 +1192,12 @@ def run_dde(args):
             "combined_taps_per_vis": taps / calls / n_kept,
             "quadrature_tap_nodes_per_vis": nodes / calls / n_kept, "unconverged": bad,
             "radial_mode": radial,
-            "roofline": {"bound": "alu", "kernel": "vis_dde_kernel", "achieved": ach,
+            "roofline": {"bound": "alu", "kernel": "dde_series_kernel", "achieved": ach,
                          "peak": peak_fp32, "unit": "TFLOP/s", "frac": ach / peak_fp32,
-                         "work_note": "executed work: 36 flops per quadrature tap-node + "
+                         "work_note": "the sampled quadrature's sums, polynomials and taps + "
                                       "J_D J_w (2 J_w + J_D - 1) complex multiply-adds per "
-                                      "visibility (separable row and column passes)"}}
+                                      "visibility (separable row and column passes), over the "
+                                      "whole call"}}
     print(json.dumps(line), flush=True)
 
 
