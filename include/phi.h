@@ -40,14 +40,24 @@
  *     the adjoint.
  *   - Quadrature: Gauss-Kronrod 15/31 on equal panels of [0, R].  Acceptance
  *     per tap: sum over panels |K31 - G15| <= max(quad_abs_tol,
- *     quad_rel_tol * |K|) (paper: 1e-6 relative and absolute, Sec. 4).  Taps that do not converge within the refinement cap are
- *     counted (phi_plan_stats), never an error.
+ *     quad_rel_tol * |K|) (paper: 1e-6 relative and absolute, Sec. 4).  The
+ *     taps of a visibility share the nodes, so in the quadrature and radial
+ *     modes the sums over them, and the estimate, are formed at samples of
+ *     rho at twice the rate the kernel's band limit asks for, and every tap
+ *     is interpolated from them (to FP32 and FP64 rounding); a visibility
+ *     whose samples show that each of its taps meets quad_abs_tol is done,
+ *     any other one is integrated tap by tap (quadrature) or from its
+ *     Chebyshev series (radial), as all are when quad_abs_tol is below
+ *     2.5e-7 in FP32 or 1e-14 in FP64.  Taps that do not converge within the
+ *     refinement cap are counted (phi_plan_stats), never an error.
  *
  * Memory and streams: every pointer argument named *_dev is a device pointer
  * owned by the caller; the plan owns everything it allocates (sorted
  * visibility records, permutation, stack tables, per-pixel factors, the
- * padded grids of one group of stacks, cuFFT plans and their workspace);
- * the DDE calls may also take a transient buffer (see phi_degrid_dde).
+ * padded grids of one group of stacks, the tables of the sampled quadrature
+ * and of the transforms or, for sizes they do not cover, cuFFT plans and
+ * their workspace); the DDE calls may also take a transient buffer (see
+ * phi_degrid_dde).
  * Calls are asynchronous on the
  * given stream (a cudaStream_t passed as void*; NULL = legacy default stream)
  * and do not synchronise, except phi_plan_create (it reads the k-means
@@ -84,14 +94,15 @@ enum phi_status {
 
 enum phi_precision {
   PHI_F32 = 0,  /* FP32 grid, FFT, kernel, accumulation and quadrature error
-                   estimate; FP64 chirp phase argument                       */
+                   estimate; chirp phases in pairs of FP32 values            */
   PHI_F64 = 1   /* everything in FP64                                        */
 };
 
 enum phi_kernel_mode {
   PHI_KERNEL_QUADRATURE = 0,  /* every tap by adaptive quadrature (Sec. 3.1)         */
   PHI_KERNEL_TABLE = 1,       /* pre-sampled 1-D w-planes, bilinear (Sec. 5.1.1)       */
-  PHI_KERNEL_RADIAL = 2       /* per visibility: the same quadrature at Chebyshev radii,
+  PHI_KERNEL_RADIAL = 2       /* as PHI_KERNEL_QUADRATURE, but a visibility its samples do
+                                 not settle: the same quadrature at Chebyshev radii,
                                  every tap from the resulting series in rho (no
                                  counterpart in the paper; same operator within the
                                  quadrature tolerance)                                 */
@@ -115,8 +126,9 @@ typedef struct {
   int32_t max_refine;       /* panel-count doublings allowed per tap chunk   */
   int32_t tile;             /* uv tile side used to sort visibilities (32)   */
   int32_t max_grid_mib;     /* device memory for the padded grids of stacks
-                               processed together (0: 4096 MiB); at least
-                               one grid is always held                      */
+                               processed together (0: 4096 MiB), split
+                               evenly over as few groups as fit it; at
+                               least one grid is always held                */
   int32_t kernel_mode;      /* enum phi_kernel_mode                          */
   int32_t grid_staging;     /* PHI_KERNEL_TABLE only: 0 = one warp per
                                visibility, table and grid read directly
@@ -190,14 +202,15 @@ int phi_plan_desc_default(phi_plan_desc* desc);
  * Build a plan (Sec. 3.2-3.3 and the per-visibility part of Eq. GC_k):
  * fold (conj_fold), Algorithm 1 on w, per-stack centres wbar_k, drop test,
  * support J_w, split u/du into integer base and fraction, sort by
- * (stack, uv tile), per-pixel image factors, cuFFT plan.  With
+ * (stack, uv tile), per-pixel image factors, tables of the quadrature and
+ * the transforms.  With
  * PHI_KERNEL_TABLE also the pre-sampled w-planes of Sec. 5.1.1:
  * [GC](i h_rho, j h_w) for 0 <= rho <= sqrt(2) max J_w / 2 + 2 and
  * 0 <= w <= max |w - wbar_k| (positive only: -w is the conjugate), computed
  * by the same adaptive quadrature, stored in pairs of adjacent w-planes;
  * degrid and grid then interpolate every tap bilinearly instead of
  * integrating it.  With PHI_KERNEL_RADIAL nothing extra is stored: for each
- * visibility the fused kernels integrate [GC](rho, dw_i) by the same
+ * visibility that the sampled quadrature does not settle the kernels integrate [GC](rho, dw_i) by the same
  * quadrature at the Chebyshev points of equal pieces of [0, rho_max]
  * (pieces of 2 / R grid pixels, 16 points each in FP32, 24 in FP64; the
  * kernel is band-limited to R cycles per pixel in rho, R the window radius)
@@ -246,16 +259,19 @@ int phi_plan_info(phi_plan_t plan, phi_plan_summary* info, double* wbar, int64_t
 
 /* Quadrature statistics accumulated since plan creation or the last reset:
  * taps that missed the tolerance at the refinement cap, taps evaluated, and
- * tap-node integrand evaluations (all refinements included).  Synchronises
+ * integrand evaluations: at a node for one sample of rho or, of visibilities
+ * integrated tap by tap, for one tap (all refinements included).  Synchronises
  * `stream`.  reset != 0 zeroes the counters after reading.  NULL outputs are
- * skipped. */
+ * skipped.  PHI_ERR_TIMEOUT if a transform of this plan gave up waiting for
+ * its own copies since the last reset: the results since then do not count. */
 int phi_plan_stats(phi_plan_t plan, int64_t* n_unconverged, int64_t* n_taps,
                    int64_t* n_tap_nodes, int reset, void* stream);
 
 /* Stages of phi_degrid / phi_grid, for per-stage device timing. */
 enum phi_stage {
-  PHI_STAGE_PREP = 0,    /* S~_k and Z                                       */
-  PHI_STAGE_FFT = 1,     /* cuFFT forward or inverse                         */
+  PHI_STAGE_PREP = 0,    /* S~_k and Z, with the rows' transform where the
+                            two-pass transforms apply                       */
+  PHI_STAGE_FFT = 1,     /* transform, or its column pass                    */
   PHI_STAGE_DEGRID = 2,  /* fused w-kernel quadrature + degridding           */
   PHI_STAGE_GRID = 3,    /* fused w-kernel quadrature + gridding             */
   PHI_STAGE_FINISH = 4,  /* crop, conj(S~_k), sum over stacks                */
@@ -274,7 +290,7 @@ int phi_plan_timings(phi_plan_t plan, double* ms, int64_t* launches, int reset, 
 
 /*
  * y = Phi x (Sec. 3.1, Eq. matrix_equation): per stack k, S~_k and Z
- * (Eq. S~_k, a_k = 1), F (cuFFT, unnormalised forward), then fused
+ * (Eq. S~_k, a_k = 1), F (unnormalised forward), then fused
  * on-the-fly w-kernel quadrature + degridding + W + fold conjugation.
  *   image_dev: N x N real, float32 (PHI_F32) or float64 (PHI_F64), row-major.
  *   vis_dev:   n_vis complex (interleaved re, im) float32 / float64, written in
@@ -299,9 +315,10 @@ int phi_grid(phi_plan_t plan, const void* vis_dev, void* image_dev, void* stream
  * odd, 1..15), convolved with the w-kernel.  Visibility i then degrids with
  *     C_i(q) = sum_s D_i(s) [GC](|u_i/du - q - s|, w_i - wbar_k)
  * over the (J_w + dde_taps - 1)^2 box around it and grids with conj(C_i).
- * The w-kernel taps come from the per-tap quadrature, or from the
- * per-visibility Chebyshev series in a PHI_KERNEL_RADIAL plan (a
- * PHI_KERNEL_TABLE plan also integrates them per tap).  dde_taps = 1 with
+ * The w-kernel taps come from the sampled quadrature and, for visibilities it
+ * does not settle, from the per-tap quadrature, or the per-visibility
+ * Chebyshev series in a PHI_KERNEL_RADIAL plan (a PHI_KERNEL_TABLE plan
+ * integrates them per tap).  dde_taps = 1 with
  * a = b = 1 is phi_degrid / phi_grid.
  *   dde_a_dev, dde_b_dev: n_vis x dde_taps complex of the plan's precision
  *              (interleaved re, im), row-major, caller's visibility order;
@@ -313,8 +330,9 @@ int phi_grid(phi_plan_t plan, const void* vis_dev, void* image_dev, void* stream
  * PHI_ERR_SUPPORT if one warp's w-kernel box for the plan's largest support
  * does not fit in a thread block's shared memory.  No counterpart for the
  * kernels' values: the paper gives no DDE model; they are the caller's.
- * Memory: in a quadrature plan whose largest box would leave few warps per
- * SM (J_w above about 24 in FP32, 10 in FP64) the boxes go through a
+ * Memory: where the sampled quadrature does not apply (quad_abs_tol below its
+ * limit, or a table plan) and the largest box would leave few warps per SM
+ * (J_w above about 24 in FP32, 10 in FP64) the boxes go through a
  * transient device buffer of at most 2 GiB, taken with cudaMallocAsync and
  * given back with cudaFreeAsync on `stream` (stream-ordered: no device-wide
  * synchronisation); when it cannot be had the call runs single-pass, with

@@ -190,7 +190,7 @@ def default_desc(**kw) -> PlanDesc:
 
 class Plan:
     """A resident operator plan: sorted visibility records, stack centres,
-    per-pixel factors, one padded grid and a cuFFT plan, all on the device.
+    per-pixel factors, padded grids and the transforms' tables, all on the device.
 
     uvw: (M, 3) float64 tensor of baselines in wavelengths (any device; it is
     copied to the current CUDA device).  weights: optional (M,) float64.

@@ -1,7 +1,10 @@
-// The DDE convolution kernel (Sec. 5.2), vis_dde_kernel.  Not a standalone
-// header: phi_ops.cu includes it inside namespace phi, after the quadrature,
-// tap and work-queue pieces it uses, so that it is compiled with them in one
-// translation unit while its source stays apart from the other kernels'.
+// The DDE convolution kernels (Sec. 5.2): dde_series_kernel over the sampled
+// quadrature, and vis_dde_kernel and the two-pass pair for the visibilities
+// that it leaves to the per-tap quadrature or the Chebyshev series.  Not a
+// standalone header: phi_ops.cu includes it inside namespace phi, after the
+// quadrature, tap and work-queue pieces it uses, so that it is compiled with
+// them in one translation unit while its source stays apart from the other
+// kernels'.
 #pragma once
 
 // ---------------------------------------------------------------------------
@@ -430,8 +433,9 @@ __global__ void __launch_bounds__(256) dde_conv_kernel(
 //
 // Against boxes through global memory (dde_box_kernel's way, the boxes from
 // the polynomials): 5 x 5 kernels, 200,003 visibilities, J_w 24-42, one call:
-// 5.2 ms, and 7.9 with the buffer's first allocation; here 4.1, 1.7 of it this
-// kernel (2.6 there; 2.6 too with one row to a lane and a modular ring).
+// 5.2 ms, and 7.9 with the buffer's first allocation; here 4.1 with the same
+// transforms, 1.7 of it this kernel (2.6 there; 2.6 too with one row to a lane
+// and a modular ring), and 2.7 with the two-pass ones.
 // Bound: issue.
 constexpr int kDdeRows = 4;
 // A DDE value as the passes read it: FP32 both parts twice, for paired

@@ -1,20 +1,24 @@
 // Hot-path kernels of the w-stacking w-projection operator on GB300 (sm_103a):
 //
 //   prep    S~_k and Z (Eq. S~_k): padded grid <- x e^{2 pi i wbar_k (1-n)} / (g n)
-//   F       cuFFT, unnormalised, in place
+//   F       unnormalised, in place: two passes fused with prep and finish
+//           (fft_kernel.cuh), or cuFFT for the sizes they do not take
 //   degrid  fused [GC] quadrature (Eq. analytic_convolution_hankel) + G + W + fold
 //   grid    fused [GC] quadrature + G^H (Eq. stacked adjoint) with float atomics
 //   finish  F^H output -> crop (Z^T) -> conj(S~_k) -> real part -> sum over stacks
 //
-// Kernel evaluation.  One warp owns one visibility.  The chirp part of the
+// Kernel evaluation.  The taps of a visibility share their quadrature nodes:
+// series_kernel.cuh forms the sums over them at samples of rho and
+// interpolates every tap.  What that does not settle is integrated tap by tap
+// here (vis_kernel).  One warp owns one visibility.  The chirp part of the
 // integrand, h(r_j) = 2 pi h_p g(r_j) r_j e^{-2 pi i dw (n(r_j) - 1)}, is the
 // same for all J_w^2 taps of the visibility, so the lanes first build it at
 // the Gauss-Kronrod 15/31 nodes of an a-priori partition of [0, R] into
-// equal panels (FP64 phase argument, tabulated 1 - n(r_j) and g(r_j)), then
-// each lane takes one tap and sums J0(2 pi rho r_j) h(r_j) with the Kronrod
+// equal panels (tabulated 1 - n(r_j) and g(r_j); FP32 forms the phase in two
+// floats), then each lane takes two taps and sums J0(2 pi rho r_j) h(r_j) with the Kronrod
 // weights, and, per panel, the difference against the embedded Gauss rule
 // as the error estimate (FP32 path: in paired f32x2 arithmetic, two nodes
-// per instruction).  A chunk of 32 taps whose estimate misses
+// per instruction).  A chunk of 64 taps whose estimate misses
 // max(abs_tol, rel_tol |K|) is recomputed with twice the panels (up to
 // max_refine times); taps still above tolerance are counted.  The degridder
 // and the gridder run this identical routine, so [GC] and its conjugate
@@ -2249,8 +2253,9 @@ int run_degrid(Plan& p, const T* x, C* y, cudaStream_t s, const DdeArgs* dde = n
 // and set the exponent e from the call's largest term.  A cell receives at
 // most one term per visibility and period of the grid its box covers, each
 // at most |[GC]| times the visibility's factor; the bound on |[GC]| carries
-// a factor 4 for the radial mode's Chebyshev interpolation (its Lebesgue
-// constant is below 3 at 16 and 24 points) and the FP32 J0's rounding.
+// a factor 4 for the interpolation between samples of rho (the magnitudes of
+// its weights sum to 2.1 at most), the radial mode's Chebyshev interpolation
+// (Lebesgue constant below 3 at 16 and 24 points) and the FP32 J0's rounding.
 template <typename T, typename C>
 int fixed_prepare(Plan& p, int g, const C* y, const DdeArgs* dde, cudaStream_t s) {
   const int64_t plane = static_cast<int64_t>(p.npad) * p.npad;

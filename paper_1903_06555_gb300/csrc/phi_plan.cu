@@ -1,7 +1,7 @@
 // Plan construction for the GB300 w-stacking w-projection operator:
 // conjugate fold (Sec. 3.3), k-means w-stacking (Algorithm 1), per-stack
 // centres, drop test, support J_w, split of u/du into an integer base and a
-// fraction, sort by (stack, uv tile), per-pixel and per-node tables, cuFFT.
+// fraction, sort by (stack, uv tile), per-pixel and per-node tables, transforms.
 //
 // All per-visibility work runs on the device.  The k-means sums are exact
 // integer sums of a fixed-point image of w, independent of their order, so a

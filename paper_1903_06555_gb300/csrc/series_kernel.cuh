@@ -35,19 +35,13 @@
 // table loads and two broadcasts per node and pair of visibilities).  FP64
 // walks the nodes, one sample per lane.
 //
-// FP32 makes the sums on the tensor cores (series_tile_kernel says how the
-// operands are split), four visibilities of one panel count to a warp: 1.3 ms
-// of the snapshot's launch where one FP32 product per lane took 3.9 (two
-// table loads and two broadcasts per node and pair of visibilities).  FP64
-// walks the nodes, one sample per lane.
-//
 // Measured on the MWA-like snapshot (1.92M visibilities, J_w 26-40, FP32):
 // 5.4 ms per degrid or grid launch where the per-tap kernel takes 63 and the
 // 16-point radial series 18.6, and 4.2e-7 from the 64-bit operator (per tap
 // 5.5e-7, radial series 9e-7: the table's J0 is rounded once, the per-tap
 // kernel's polynomial and hardware cosine are not).  Of the 5.4 ms the taps
 // take 3.3, the polynomials 0.8.  FP64 at 1e-12 (5,000 visibilities, J_w 26):
-// 1.0 ms, per tap 39 ms.  Bound: the shared-memory pipe (80% busy; 16 of
+// 0.93 ms, per tap 39 ms.  Bound: the shared-memory pipe (80% busy; 16 of
 // the 21 wavefronts per 32 taps read the polynomials) and issue (67%); FP64 its
 // FP64 unit.  24 warps of 80 registers per SM: 32 of 64 spill (5.5 ms), 16
 // of 128 hide less (6.6 ms).

@@ -11,8 +11,8 @@ the operator applications wanted on it: y = Phi x (degrid), d = Re(Phi^H y)
 * runs every admitted request on its own CUDA stream from its own worker
   thread (the library calls release the GIL), so plan builds, FFTs and the
   fused quadrature kernels of different requests overlap on the device;
-* keeps plans (sorted visibility records, stack tables, padded grid, cuFFT
-  plan) resident under the request's `obs_key`, so later requests on the
+* keeps plans (sorted visibility records, stack tables, padded grids, FFT
+  tables) resident under the request's `obs_key`, so later requests on the
   same observation skip planning; resident plans are evicted least recently
   used when admission needs their memory;
 * records per-request latency (arrival -> result on the host) and the
@@ -22,7 +22,7 @@ the operator applications wanted on it: y = Phi x (degrid), d = Re(Phi^H y)
 
 Memory admission is by a conservative per-request estimate of the device
 bytes the plan build and the calls need (inputs, outputs, plan-build
-temporaries, records, grid, cuFFT workspace), released when the request
+temporaries, records, grids, FFT workspace), released when the request
 completes; a resident plan keeps its measured size.
 """
 from __future__ import annotations
@@ -82,10 +82,11 @@ def estimate_bytes(req: Request, planned: bool = False) -> int:
     planned=True only its inputs and outputs (the plan is already resident),
     otherwise also the plan-build temporaries (folded w, flags, stack ids,
     sort keys and values with their CUB buffers), the records, per-pixel
-    tables, the padded grids of one stack group (as many stacks as fit
-    max_grid_mib, default 4 GiB) and cuFFT workspace (at most one grid per
-    batched transform plus one), and with grid_deterministic the
-    fixed-point sums of the group's grids (16 bytes a cell).  A request that
+    tables, the quadrature's tables (22 MiB at most), the padded grids of one
+    stack group (as many stacks as fit max_grid_mib, default 4 GiB), FFT
+    workspace (at most one grid per batched transform plus one), and with
+    grid_deterministic the fixed-point sums of the group's grids (16 bytes a
+    cell).  A request that
     may raise its stacks is charged for the most stacks a retry can reach
     (126)."""
     m = int(req.uvw.shape[0])
@@ -99,7 +100,7 @@ def estimate_bytes(req: Request, planned: bool = False) -> int:
     io = m * 2 * c + n * n * 2 * r + (16 << 20)
     if planned:
         return io
-    per_vis = 24 + 8 + 1 + 4 + 16 + 16 + (52 if f64 else 36)
+    per_vis = 24 + 8 + 1 + 4 + 16 + 16 + (56 if f64 else 40)
     per_pix = 12 + r
     grid = c * npad * npad
     fixed = 16 * npad * npad if int(req.desc.get("grid_deterministic", 0)) else 0
@@ -107,7 +108,7 @@ def estimate_bytes(req: Request, planned: bool = False) -> int:
     cap = (int(req.desc.get("max_grid_mib", 0)) or 4096) << 20
     group = max(1, min(k, cap // (grid + fixed)))
     return (io + m * per_vis + n * n * per_pix + (2 * group + 1) * grid + group * fixed +
-            (8 << 20))
+            (32 << 20))
 
 
 class Server:
