@@ -585,7 +585,7 @@ __global__ void fixed_to_grid_kernel(const longlong2* __restrict__ cells,
 
 // Build the weighted integrand values for panels [p0, p0 + np) of the
 // npan-panel partition: h(r_j) e^{2 pi i dw (1 - n(r_j))}, phase argument in
-// FP64, one NodeVal per node (FP64 path: Kronrod and difference weights).
+// FP64 or two floats, one NodeVal per node (FP64 path: Kronrod and difference weights).
 template <typename T>
 __device__ __forceinline__ void build_nodes(NodeVal<T>* sh, const QuadParams& q, int npan, int p0,
                                             int np, double dw, int lane) {
@@ -1572,15 +1572,20 @@ __global__ void __launch_bounds__(256) row_table_kernel(
   flush_counts(stats, 0, my_taps, 0, lane);
 }
 
+// j0_hc of two arguments in paired arithmetic.
+__device__ __forceinline__ float2 j0_hc2(float2 u) {
+  return fminf(u.x, u.y) > kJ0Split ? j0_pair_regime<kPairNear>(u) : j0_pair_regime<kPairBoth>(u);
+}
+
 // [GC] at arbitrary points (phi_wkernel and phi_wkernel_noalloc): every point
 // has its own |dw|, so nothing but the node table is shared.  L lanes take a
 // point, each the nodes k = sub, sub + L, ... of every panel, with the node
-// value and J0 formed together; per panel two shuffles over the L lanes make
-// the Kronrod-minus-Gauss sum for the estimate, refined as eval_chunk does
-// for a chunk of one tap.  (One warp per point, all lanes at the one tap,
-// repeated every Bessel function 32 times: 113 us for 40,009 points in FP32.)
-// Bound: FP32 issue, ~90 instructions per node.  L = 4 keeps the shuffles
-// below a tenth of that; 32 when there are too few points to fill the chip.
+// value and J0 formed together, FP32 two nodes at a time in paired arithmetic;
+// per panel two shuffles over the L lanes make the Kronrod-minus-Gauss sum for
+// the estimate, refined as eval_chunk does for a chunk of one tap.  (One warp
+// per point, all lanes at the one tap, repeated every Bessel function 32
+// times: 113 us for 40,009 points in FP32; L = 4 node by node: 30.8.)  Bound:
+// FP32 issue and the longest of a warp's points, FP64 its FP64 unit.
 template <typename T, typename C, int L>
 __device__ __forceinline__ void wkernel_points(const double* __restrict__ rho_in,
                                                const double* __restrict__ dw_in, int64_t n,
@@ -1606,26 +1611,50 @@ __device__ __forceinline__ void wkernel_points(const double* __restrict__ rho_in
       for (int p = 0; p < npan; ++p) {
         const T a = Bh * static_cast<T>(2 * p + 1);
         T dr = 0, di = 0;
+        if constexpr (sizeof(T) == 4) {
+          const float* hks = static_cast<const float*>(q.node_hk) + off + kNodes * p;
+          const float* hds = static_cast<const float*>(q.node_hd) + off + kNodes * p;
+          const float2* oms = q.node_omn2 + off + kNodes * p;
+          float2 r2 = make_float2(kr, 0.0f), i2 = make_float2(ki, 0.0f);
+          float2 dr2 = make_float2(0.0f, 0.0f), di2 = dr2;
 #pragma unroll 1
-        for (int k = sub; k < kNodes; k += L) {
-          const int64_t j = off + kNodes * p + k;
-          const T hk = static_cast<const T*>(q.node_hk)[j];
-          T hd = static_cast<const T*>(q.node_hd)[j];
-          C e;
-          if constexpr (sizeof(T) == 4) {
-            hd = hk - hd;   // FP32 tabulates the Gauss weight, FP64 the difference
-            const float2 om = q.node_omn2[j];
-            e = phase(om.x, om.y);
-          } else {
+          for (int k = sub; k < kNodes; k += 2 * L) {
+            const bool both = k + L < kNodes;
+            const int m = both ? k + L : k;
+            const float2 om = oms[k], om2 = oms[m];
+            const float2 e = phase(om.x, om.y), e2 = phase(om2.x, om2.y);
+            const float2 hk = make_float2(hks[k], both ? hks[m] : 0.0f);
+            const float2 hg = make_float2(hds[k], both ? hds[m] : 0.0f);
+            const float2 J = j0_hc2(__ffma2_rn(make_float2(Bh, Bh),
+                                               make_float2(gk_node_c(T(0), k), gk_node_c(T(0), m)),
+                                               make_float2(a, a)));
+            const float2 Jk = __fmul2_rn(J, hk);
+            const float2 Jd = __fmul2_rn(J, __fadd2_rn(hk, make_float2(-hg.x, -hg.y)));
+            const float2 c = make_float2(e.x, e2.x), s2 = make_float2(e.y, e2.y);
+            r2 = __ffma2_rn(Jk, c, r2);
+            i2 = __ffma2_rn(Jk, s2, i2);
+            dr2 = __ffma2_rn(Jd, c, dr2);
+            di2 = __ffma2_rn(Jd, s2, di2);
+          }
+          kr = r2.x + r2.y;
+          ki = i2.x + i2.y;
+          dr = dr2.x + dr2.y;
+          di = di2.x + di2.y;
+        } else {
+#pragma unroll 1
+          for (int k = sub; k < kNodes; k += L) {
+            const int64_t j = off + kNodes * p + k;
+            const T hk = static_cast<const T*>(q.node_hk)[j], hd = static_cast<const T*>(q.node_hd)[j];
             double t = dw * q.node_omn[j];
             t -= rint(t);
+            C e;
             sincos_pi(2.0 * t, &e.y, &e.x);
+            const T J = j0_hc(fma(Bh, gk_node_c(T(0), k), a));
+            kr = fma(J * hk, e.x, kr);
+            ki = fma(J * hk, e.y, ki);
+            dr = fma(J * hd, e.x, dr);
+            di = fma(J * hd, e.y, di);
           }
-          const T J = j0_hc(fma(Bh, gk_node_c(T(0), k), a));
-          kr = fma(J * hk, e.x, kr);
-          ki = fma(J * hk, e.y, ki);
-          dr = fma(J * hd, e.x, dr);
-          di = fma(J * hd, e.y, di);
         }
 #pragma unroll
         for (int o = L / 2; o > 0; o >>= 1) {
@@ -1659,19 +1688,25 @@ __global__ void __launch_bounds__(256) wkernel_kernel(const double* __restrict__
   wkernel_points<T, C, L>(rho_in, dw_in, n, out, q, max_panels, bad);
 }
 
-// Four lanes per point once that gives every SM two warps or more, a warp
-// per point below.
+// Lanes per point.  Many are soon done with a point, few waste less on its
+// shuffles.  FP32, 16 against 4: 8.9 and 16.0 us for 5,000 points, 23.9 and
+// 27.9 for 40,009, 49 and 50 for 100,000, 172 and 162 for 400,000.  FP64 (31
+// nodes of its slow J0 in one pass of a warp), 32 against 4: 0.34 and 0.59 ms
+// for 8,000, 6.7 and 8.8 ms for 200,000.
 template <typename T, typename C>
 cudaError_t launch_wkernel(const double* rho, const double* dw, int64_t n, C* out,
                            const QuadParams& q, int max_panels, unsigned long long* bad,
                            int num_sms, cudaStream_t s) {
-  const bool wide = n < 16 * (int64_t)num_sms;
-  const int64_t want = (n * (wide ? 32 : 4) + 255) / 256;
-  const int blocks = static_cast<int>(std::min<int64_t>(want, 65535));
-  if (wide)
+  const bool many = n >= 640 * (int64_t)num_sms;
+  const int lanes = sizeof(T) == 8 ? 32 : many ? 4 : 16;
+  const int blocks = static_cast<int>(std::min<int64_t>((n * lanes + 255) / 256, 65535));
+  if constexpr (sizeof(T) == 8) {
     wkernel_kernel<T, C, 32><<<blocks, 256, 0, s>>>(rho, dw, n, out, q, max_panels, bad);
-  else
+  } else if (many) {
     wkernel_kernel<T, C, 4><<<blocks, 256, 0, s>>>(rho, dw, n, out, q, max_panels, bad);
+  } else {
+    wkernel_kernel<T, C, 16><<<blocks, 256, 0, s>>>(rho, dw, n, out, q, max_panels, bad);
+  }
   return cudaGetLastError();
 }
 
