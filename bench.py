@@ -220,7 +220,7 @@ def kernel_source_hash():
     import hashlib
     h = hashlib.sha256()
     for f in ("phi_ops.cu", "bessel_j0.cuh", "phi_internal.cuh", "table_index.cuh",
-              "fixed_point.cuh", "series_kernel.cuh", "series_coef.cuh", "fft_kernel.cuh"):
+              "fixed_point.cuh", "series_kernel.cuh", "series_coef.cuh", "fft_kernel.cuh", "czt_kernel.cuh"):
         with open(os.path.join(ROOT, "paper_1903_06555_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

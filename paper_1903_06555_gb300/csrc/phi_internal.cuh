@@ -198,8 +198,9 @@ struct Plan {
   double* wbar_dev = nullptr;
   cufftHandle fft_batch = 0;            // fft_batch_n transforms in one call
   int fft_batch_n = 1;
-  int fft_log = 0;                      // two-pass transforms: log2 N (0: cuFFT)
-  void* fft_tab = nullptr;              // their roots of unity
+  int fft_log = 0;                      // two-pass transforms: log2 N, or 0
+  int czt_log = 0;                      // chirp transforms: log2 of their length, or 0
+  void* fft_tab = nullptr;              // their roots of unity and chirp (neither: cuFFT)
   FftMaps fft_maps;
   bool fft_batch_ok = false;
   // [0..K) work heads, [K] unconverged taps, [K+1] taps, [K+2] wkernel misses,
@@ -321,7 +322,8 @@ int build_kernel_table(Plan& p, cudaStream_t s);
 int build_radial_tables(Plan& p, cudaStream_t s);
 int build_series_tables(Plan& p, cudaStream_t s);
 int fft_two_pass_log(int N, int npad, bool f64);   // log2 N where the two-pass transforms apply, or 0
-int fft_two_pass_table(int N);           // complex values of their table
+int chirp_log(int N, int npad, bool f64);          // log2 M where the chirp transforms apply, or 0
+int64_t own_transform_table(const Plan& p);        // complex values of the plan's transform table
 int build_fft_table(Plan& p, cudaStream_t s);
 int compute_kernel_bound(Plan& p, double* scratch, cudaStream_t s);  // scratch: kMaxPanels doubles
 

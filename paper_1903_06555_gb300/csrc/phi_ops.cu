@@ -2,7 +2,7 @@
 //
 //   prep    S~_k and Z (Eq. S~_k): padded grid <- x e^{2 pi i wbar_k (1-n)} / (g n)
 //   F       unnormalised, in place: two passes fused with prep and finish
-//           (fft_kernel.cuh), or cuFFT for the sizes they do not take
+//           (fft_kernel.cuh, czt_kernel.cuh), or cuFFT for the other sizes
 //   degrid  fused [GC] quadrature (Eq. analytic_convolution_hankel) + G + W + fold
 //   grid    fused [GC] quadrature + G^H (Eq. stacked adjoint) with float atomics
 //   finish  F^H output -> crop (Z^T) -> conj(S~_k) -> real part -> sum over stacks
@@ -489,6 +489,7 @@ __global__ void finish_kernel(const C* __restrict__ grids,
 
 // The image-domain steps and the FFTs in two passes, for N = 2^6 .. 2^11, os 2
 #include "fft_kernel.cuh"
+#include "czt_kernel.cuh"
 
 // ---------------------------------------------------------------------------
 // Deterministic gridding: fixed-point grid sums
@@ -2142,6 +2143,7 @@ struct DdeArgs {
 
 // launch_fft_forward, launch_fft_adjoint
 #include "fft_launch.cuh"
+#include "czt_launch.cuh"
 
 // launch_series, dde_warp_smem, launch_dde
 #include "series_launch.cuh"
@@ -2218,15 +2220,25 @@ int launch_group_kernel(Plan& p, int g, const C* grids_in, C* grids_out, const C
   return PHI_OK;
 }
 
-// S~_k, Z and F for the n grids of group g: the two-pass transforms where
-// they take the grid (the row pass timed as prep, the column pass as FFT),
-// prep and cuFFT otherwise.
+// The transforms of fft_kernel.cuh or czt_kernel.cuh (FP32) where they apply.
+bool own_transform(const Plan& p) { return p.fft_log || p.czt_log; }
+template <typename T, typename C>
+int own_pass(Plan& p, FftPass pass, const int32_t* stacks, int n, const T* x_in, C* grids,
+             T* x_out, int accumulate, cudaStream_t s) {
+  if constexpr (sizeof(T) == 4)
+    if (p.czt_log) return czt_pass(p, pass, stacks, n, x_in, grids, x_out, accumulate, s);
+  return fft_pass<T, C>(p, pass, stacks, n, x_in, grids, x_out, accumulate, s);
+}
+
+// S~_k, Z and F for the n grids of group g: our transforms where they take the
+// grid (the row pass timed as prep, the column pass as FFT), prep and cuFFT
+// otherwise.
 template <typename T, typename C>
 int image_to_grids(Plan& p, int g, int n, const T* x, C* grids, cudaStream_t s) {
   const int32_t* stacks = p.group_stacks_dev + p.group_off[g];
   long ev = timer_begin(p, s);
-  if (p.fft_log) {
-    PHI_TRY_ST((fft_pass<T, C>(p, kFftRowsForward, stacks, n, x, grids, nullptr, 0, s)));
+  if (own_transform(p)) {
+    PHI_TRY_ST((own_pass<T, C>(p, kFftRowsForward, stacks, n, x, grids, nullptr, 0, s)));
   } else {
     prep_kernel<T, C><<<dim3(p.num_sms * 4, n), 256, 0, s>>>(
         x, static_cast<const typename PixelPhase<T>::omn*>(p.omn_pix),
@@ -2235,8 +2247,8 @@ int image_to_grids(Plan& p, int g, int n, const T* x, C* grids, cudaStream_t s) 
   }
   timer_end(p, ev, PHI_STAGE_PREP, s);
   ev = timer_begin(p, s);
-  if (p.fft_log)
-    PHI_TRY_ST((fft_pass<T, C>(p, kFftColsForward, stacks, n, x, grids, nullptr, 0, s)));
+  if (own_transform(p))
+    PHI_TRY_ST((own_pass<T, C>(p, kFftColsForward, stacks, n, x, grids, nullptr, 0, s)));
   else
     PHI_TRY_ST((fft_group<T, C>(p, grids, n, CUFFT_FORWARD, s)));
   timer_end(p, ev, PHI_STAGE_FFT, s);
@@ -2248,14 +2260,14 @@ template <typename T, typename C>
 int grids_to_image(Plan& p, int g, int n, C* grids, T* x, cudaStream_t s) {
   const int32_t* stacks = p.group_stacks_dev + p.group_off[g];
   long ev = timer_begin(p, s);
-  if (p.fft_log)
-    PHI_TRY_ST((fft_pass<T, C>(p, kFftColsAdjoint, stacks, n, nullptr, grids, nullptr, 0, s)));
+  if (own_transform(p))
+    PHI_TRY_ST((own_pass<T, C>(p, kFftColsAdjoint, stacks, n, nullptr, grids, nullptr, 0, s)));
   else
     PHI_TRY_ST((fft_group<T, C>(p, grids, n, CUFFT_INVERSE, s)));
   timer_end(p, ev, PHI_STAGE_FFT, s);
   ev = timer_begin(p, s);
-  if (p.fft_log) {
-    PHI_TRY_ST((fft_pass<T, C>(p, kFftRowsAdjoint, stacks, n, nullptr, grids, x, g == 0 ? 0 : 1, s)));
+  if (own_transform(p)) {
+    PHI_TRY_ST((own_pass<T, C>(p, kFftRowsAdjoint, stacks, n, nullptr, grids, x, g == 0 ? 0 : 1, s)));
   } else {
     finish_kernel<T, C><<<p.num_sms * 4, 256, 0, s>>>(
         grids, static_cast<const typename PixelPhase<T>::omn*>(p.omn_pix),
@@ -2379,9 +2391,13 @@ int build_radial_tables(Plan& p, cudaStream_t s) {
 }
 
 int fft_two_pass_log(int N, int npad, bool f64) { return fft_log(N, npad, f64); }
-int fft_two_pass_table(int N) { return fft_table_size(N); }
+int chirp_log(int N, int npad, bool f64) { return czt_log(N, npad, f64); }
+int64_t own_transform_table(const Plan& p) {
+  return p.czt_log ? czt_table_size(p.N, p.czt_log) : fft_table_size(p.N);
+}
 
 int build_fft_table(Plan& p, cudaStream_t s) {
+  if (p.czt_log) return czt_setup(p, s);
   if (p.d.precision == PHI_F64)
     PHI_TRY_ST((fft_setup<double, double2>(p)));
   else

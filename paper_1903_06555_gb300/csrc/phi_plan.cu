@@ -828,9 +828,10 @@ int build(Plan& p, const double* uvw, const double* weights, int64_t M, cudaStre
   if (d.kernel_mode == PHI_KERNEL_RADIAL) PHI_TRY(build_radial_tables(p, s));
   if (d.kernel_mode != PHI_KERNEL_TABLE) PHI_TRY(build_series_tables(p, s));
   p.fft_log = fft_two_pass_log(p.N, p.npad, f64);
-  if (p.fft_log) {
+  if (!p.fft_log) p.czt_log = chirp_log(p.N, p.npad, f64);
+  if (p.fft_log || p.czt_log) {
     PHI_CUDA_TRY(owned_alloc(p, reinterpret_cast<unsigned char**>(&p.fft_tab),
-                             2 * tsize * static_cast<size_t>(fft_two_pass_table(p.N))));
+                             2 * tsize * static_cast<size_t>(own_transform_table(p))));
     PHI_TRY(build_fft_table(p, s));
     PHI_CUDA_TRY(cudaStreamSynchronize(s));
     return PHI_OK;
