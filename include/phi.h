@@ -263,9 +263,17 @@ int phi_plan_info(phi_plan_t plan, phi_plan_summary* info, double* wbar, int64_t
  * integrated tap by tap, for one tap (all refinements included).  Synchronises
  * `stream`.  reset != 0 zeroes the counters after reading.  NULL outputs are
  * skipped.  PHI_ERR_TIMEOUT if a transform of this plan gave up waiting for
- * its own copies since the last reset: the results since then do not count. */
+ * its own copies since the last reset: every value that call computed from the
+ * columns left undone is NaN. */
 int phi_plan_stats(phi_plan_t plan, int64_t* n_unconverged, int64_t* n_taps,
                    int64_t* n_tap_nodes, int reset, void* stream);
+
+/* How often the column passes of this plan's transforms poll for a copy of
+ * theirs before they give up (phi_plan_stats), about a microsecond a poll.
+ * Plans start with 2^20, which polls < 0 or above restores; 0 makes every
+ * wait run out at once, so that a program can see what it does about it.
+ * Of no effect where the transforms do not wait (other image sizes). */
+int phi_plan_set_wait_limit(phi_plan_t plan, int polls);
 
 /* Stages of phi_degrid / phi_grid, for per-stage device timing. */
 enum phi_stage {

@@ -139,6 +139,7 @@ def lib():
             L.phi_plan_info.argtypes = [_vp, ctypes.POINTER(PlanSummary), _vp, _vp, _vp]
             L.phi_plan_stats.argtypes = [_vp, ctypes.POINTER(_i64), ctypes.POINTER(_i64),
                                          ctypes.POINTER(_i64), ctypes.c_int, _vp]
+            L.phi_plan_set_wait_limit.argtypes = [_vp, ctypes.c_int]
             L.phi_plan_set_timing.argtypes = [_vp, ctypes.c_int]
             L.phi_plan_timings.argtypes = [_vp, ctypes.POINTER(ctypes.c_double),
                                            ctypes.POINTER(_i64), ctypes.c_int, _vp]
@@ -360,6 +361,12 @@ class Plan:
         _check(lib().phi_plan_stats(self._h, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c),
                                     int(reset), _stream(stream)), "phi_plan_stats")
         return int(a.value), int(b.value), int(c.value)
+
+    def set_wait_limit(self, polls=-1):
+        """Polls of a transform's wait before it gives up (-1: the default).
+        After that the results are NaN and stats() raises PHI_ERR_TIMEOUT
+        until it is reset."""
+        _check(lib().phi_plan_set_wait_limit(self._h, int(polls)), "phi_plan_set_wait_limit")
 
     def set_timing(self, enable=True):
         _check(lib().phi_plan_set_timing(self._h, int(enable)), "phi_plan_set_timing")

@@ -347,10 +347,11 @@ __device__ __forceinline__ void fft_bar_expect(unsigned long long* bar, unsigned
                "r"(bytes)
                : "memory");
 }
-// Waits for the phase of the given parity, for at most about a second; false
-// if it did not complete (the block then records it and leaves).
-__device__ __forceinline__ bool fft_bar_wait(unsigned long long* bar, unsigned parity) {
-  for (int i = 0; i < (1 << 20); ++i) {
+// Waits for the phase of the given parity, polling `limit` times at most; false
+// if it did not complete.
+constexpr int kFftWaitLimit = 1 << 20;   // polls of about a microsecond each
+__device__ __forceinline__ bool fft_bar_wait(unsigned long long* bar, unsigned parity, int limit) {
+  for (int i = 0; i < limit; ++i) {
     unsigned done;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -362,6 +363,23 @@ __device__ __forceinline__ bool fft_bar_wait(unsigned long long* bar, unsigned p
     if (done) return true;
   }
   return false;
+}
+// What a block does about the tiles it will not transform, after its copies
+// have been waited for: it records that it gave up, and every row of those
+// tiles that the next pass reads becomes NaN, so that no result computed from
+// them passes for a value.
+template <typename T, typename C, int N, int NC>
+__device__ __noinline__ void fft_give_up(C* __restrict__ grids, int rows, int tile, int tiles,
+                                         int* __restrict__ timeout) {
+  constexpr int kTiles = 2 * N / NC;
+  if (threadIdx.x == 0) *timeout = 1;
+  C nan;
+  nan.x = nan.y = static_cast<T>(NAN);
+  for (; tile < tiles; tile += gridDim.x) {
+    C* g = grids + static_cast<int64_t>(tile / kTiles) * 4 * N * N + tile % kTiles * NC;
+    for (int i = threadIdx.x; i < rows * NC; i += blockDim.x)
+      g[static_cast<int64_t>(i / NC) * 2 * N + i % NC] = nan;
+  }
 }
 // N rows of a tile into buf: rows of the image map, or rows of one parity of
 // the half map (one thread).
@@ -425,9 +443,11 @@ __device__ __forceinline__ void fft_publish() { asm volatile("fence.proxy.async.
 template <typename T, typename C, int kLog>
 __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
     fft_cols_forward_kernel(const C* __restrict__ tab, const __grid_constant__ FftMaps maps,
-                            int tiles, int* __restrict__ timeout) {
+                            C* __restrict__ grids, int tiles, int limit,
+                            int* __restrict__ timeout) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bar;
+  __shared__ int failed;   // a thread's wait ran out; read after the next barrier
   constexpr int N = 1 << kLog, TPC = N / 16, NC = fft_cols<kLog, T>(), kTiles = 2 * N / NC;
   const int c = threadIdx.x % NC, j = threadIdx.x / NC;
   C* in = reinterpret_cast<C*>(fft_aligned(smem_raw));
@@ -435,24 +455,23 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
   C* sh = out + N * NC + c * fft_col_elems<kLog, T>();
   const bool lead = threadIdx.x == 0;
   if (lead) {
+    failed = 0;
     fft_bar_init(&bar);
     fft_tile_load<C, N, NC, false>(in, &maps, blockIdx.x % kTiles * NC, 0, blockIdx.x / kTiles, &bar);
   }
   __syncthreads();
   unsigned parity = 0;
-  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, parity ^= 1) {
+  int tile = blockIdx.x;
+  for (; tile < tiles; tile += gridDim.x, parity ^= 1) {
     const int col = tile % kTiles * NC, grid = tile / kTiles, next = tile + gridDim.x;
-    if (!fft_bar_wait(&bar, parity)) {
-      if (lead) *timeout = 1;
-      fft_bar_wait(&bar, parity);
-      break;
-    }
+    if (!fft_bar_wait(&bar, parity, limit)) failed = 1;
     C v[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) v[m] = in[((j + m * TPC) ^ (N / 2)) * NC + c];
     fft_points<kLog, -1>(v, sh, j, tab);
     if (lead) fft_stores_read();
     __syncthreads();
+    if (failed) break;   // the whole block; the tile's load is the one copy in flight
 #pragma unroll
     for (int m = 0; m < 16; ++m) out[(j + m * TPC) * NC + c] = v[m];
     fft_publish();
@@ -475,6 +494,11 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
     __syncthreads();
     if (lead) fft_tile_store<C, N, NC, true>(out, &maps, col, 1, grid);
   }
+  if (failed) {
+    if (lead) fft_bar_wait(&bar, parity, kFftWaitLimit);
+    __syncthreads();
+    fft_give_up<T, C, N, NC>(grids, 2 * N, tile, tiles, timeout);
+  }
   if (lead) fft_stores_done();
 }
 
@@ -485,9 +509,11 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
 template <typename T, typename C, int kLog>
 __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
     fft_cols_adjoint_kernel(const C* __restrict__ tab, const __grid_constant__ FftMaps maps,
-                            int tiles, int* __restrict__ timeout) {
+                            C* __restrict__ grids, int tiles, int limit,
+                            int* __restrict__ timeout) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bars[2];
+  __shared__ int failed;   // a thread's wait ran out; read after the next barrier
   constexpr int N = 1 << kLog, TPC = N / 16, NC = fft_cols<kLog, T>(), kTiles = 2 * N / NC;
   const int c = threadIdx.x % NC, j = threadIdx.x / NC;
   C* buf = reinterpret_cast<C*>(fft_aligned(smem_raw));   // even rows
@@ -496,6 +522,7 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
   C* sh = out + c * fft_col_elems<kLog, T>();
   const bool lead = threadIdx.x == 0;
   if (lead) {
+    failed = 0;
     fft_bar_init(&bars[0]);
     fft_bar_init(&bars[1]);
     const int col = blockIdx.x % kTiles * NC, grid = blockIdx.x / kTiles;
@@ -503,30 +530,26 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
     fft_tile_load<C, N, NC, true>(buf1, &maps, col, 1, grid, &bars[1]);
   }
   __syncthreads();
-  unsigned parity = 0;
-  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, parity ^= 1) {
+  unsigned parity = 0, parity0 = 0;   // parity0: of the load last sent to the even rows' buffer
+  int tile = blockIdx.x;
+  for (; tile < tiles; tile += gridDim.x, parity ^= 1) {
     const int col = tile % kTiles * NC, grid = tile / kTiles, next = tile + gridDim.x;
     C even[16], v[16];
-    if (!fft_bar_wait(&bars[0], parity)) {
-      if (lead) *timeout = 1;
-      fft_bar_wait(&bars[0], parity);
-      break;
-    }
+    if (!fft_bar_wait(&bars[0], parity, limit)) failed = 1;
 #pragma unroll
     for (int m = 0; m < 16; ++m) even[m] = buf[(j + m * TPC) * NC + c];
     if (lead) fft_stores_read();   // the exchange's memory is free again
     __syncthreads();               // and the even rows have been read
+    if (failed) break;             // the whole block
+    parity0 = next < tiles ? parity ^ 1 : parity;
     if (lead && next < tiles)
       fft_tile_load<C, N, NC, true>(buf, &maps, next % kTiles * NC, 0, next / kTiles, &bars[0]);
     fft_points<kLog, 1>(even, sh, j, tab);
-    if (!fft_bar_wait(&bars[1], parity)) {
-      if (lead) *timeout = 1;
-      fft_bar_wait(&bars[1], parity);
-      break;
-    }
+    if (!fft_bar_wait(&bars[1], parity, limit)) failed = 1;
 #pragma unroll
     for (int m = 0; m < 16; ++m) v[m] = buf1[(j + m * TPC) * NC + c];
     __syncthreads();               // the odd rows have been read
+    if (failed) break;             // the whole block
     if (lead && next < tiles)
       fft_tile_load<C, N, NC, true>(buf1, &maps, next % kTiles * NC, 1, next / kTiles, &bars[1]);
     fft_points<kLog, 1>(v, sh, j, tab);
@@ -540,6 +563,14 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
     fft_publish();
     __syncthreads();
     if (lead) fft_tile_store<C, N, NC, false>(out, &maps, col, 0, grid);
+  }
+  if (failed) {   // one load may be in flight to each buffer
+    if (lead) {
+      fft_bar_wait(&bars[0], parity0, kFftWaitLimit);
+      fft_bar_wait(&bars[1], parity, kFftWaitLimit);
+    }
+    __syncthreads();
+    fft_give_up<T, C, N, NC>(grids, N, tile, tiles, timeout);
   }
   if (lead) fft_stores_done();
 }

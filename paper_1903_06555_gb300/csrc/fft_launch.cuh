@@ -77,12 +77,12 @@ int fft_pass_log(Plan& p, FftPass pass, const int32_t* stacks, int n, const T* x
     case kFftColsForward:
       fft_cols_forward_kernel<T, C, kLog>
           <<<cols(fft_cols_forward_kernel<T, C, kLog>), col_threads, col_smem, s>>>(
-              tab, p.fft_maps, tiles, timeout);
+              tab, p.fft_maps, grids, tiles, p.fft_wait_limit, timeout);
       break;
     case kFftColsAdjoint:
       fft_cols_adjoint_kernel<T, C, kLog>
           <<<cols(fft_cols_adjoint_kernel<T, C, kLog>), col_threads, col_smem, s>>>(
-              tab, p.fft_maps, tiles, timeout);
+              tab, p.fft_maps, grids, tiles, p.fft_wait_limit, timeout);
       break;
     case kFftRowsAdjoint:
       fft_rows_adjoint_kernel<T, C, kLog><<<rows.y, row_threads, row_smem, s>>>(

@@ -202,6 +202,7 @@ struct Plan {
   int czt_log = 0;                      // chirp transforms: log2 of their length, or 0
   void* fft_tab = nullptr;              // their roots of unity and chirp (neither: cuFFT)
   FftMaps fft_maps;
+  int fft_wait_limit = 0;               // polls of a column pass's wait (set with the maps)
   bool fft_batch_ok = false;
   // [0..K) work heads, [K] unconverged taps, [K+1] taps, [K+2] wkernel misses,
   // [K+3] node evaluations, [K+4] a transform's bounded wait ran out;
@@ -325,6 +326,7 @@ int fft_two_pass_log(int N, int npad, bool f64);   // log2 N where the two-pass 
 int chirp_log(int N, int npad, bool f64);          // log2 M where the chirp transforms apply, or 0
 int64_t own_transform_table(const Plan& p);        // complex values of the plan's transform table
 int build_fft_table(Plan& p, cudaStream_t s);
+int transform_wait_limit();                        // polls a wait of the column passes takes by itself
 int compute_kernel_bound(Plan& p, double* scratch, cudaStream_t s);  // scratch: kMaxPanels doubles
 
 }  // namespace phi

@@ -2396,7 +2396,10 @@ int64_t own_transform_table(const Plan& p) {
   return p.czt_log ? czt_table_size(p.N, p.czt_log) : fft_table_size(p.N);
 }
 
+int transform_wait_limit() { return kFftWaitLimit; }
+
 int build_fft_table(Plan& p, cudaStream_t s) {
+  p.fft_wait_limit = kFftWaitLimit;
   if (p.czt_log) return czt_setup(p, s);
   if (p.d.precision == PHI_F64)
     PHI_TRY_ST((fft_setup<double, double2>(p)));

@@ -999,6 +999,13 @@ extern "C" int phi_plan_stats(phi_plan_t plan, int64_t* n_unconverged, int64_t* 
   return h[4] ? PHI_ERR_TIMEOUT : PHI_OK;
 }
 
+extern "C" int phi_plan_set_wait_limit(phi_plan_t plan, int polls) {
+  if (!plan) return PHI_ERR_ARG;
+  const int most = phi::transform_wait_limit();
+  plan->fft_wait_limit = polls < 0 || polls > most ? most : polls;
+  return PHI_OK;
+}
+
 extern "C" const char* phi_error_string(int status) {
   switch (status) {
     case PHI_OK: return "ok";

@@ -275,6 +275,8 @@ class Server:
                 if "degrid" in req.ops:
                     res.y = y.to("cpu", non_blocking=True)
                 stream.synchronize()
+                # a transform that gave up waiting says so in the plan's status only
+                plan.stats(reset=True, stream=stream)
                 if res.y is not None:
                     res.y = res.y.numpy()
                 if res.dirty is not None:
@@ -283,6 +285,7 @@ class Server:
         except (PhiError, RuntimeError, ValueError) as e:
             res.status = "error"
             res.error = str(e)
+            res.y = res.dirty = None
         res.done = self.now()
         with self._lock:
             self._in_use -= need
