@@ -576,9 +576,23 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
 }
 
 // Row pass of the adjoint: row p of every grid of the group, times conj(S~_k),
-// real part, summed over the stacks into image row p.
+// real part, summed over the stacks into image row p.  One block per row (or
+// rows: fft_rows); where the rows of a small image leave the chip idle the
+// stacks are split over `groups` sets of threads of the block (set g takes
+// stacks g, g + groups, ...), whose sums are added in the order of the sets.
+// Serial over the stacks, one warp for 8 rows of 64^2 took 1.4 us a stack (24
+// stacks 38.7 us, with the sets 15.5; 126 177 and 55; 128^2, 24 stacks, 42.6
+// and 14.7), and the whole adjoint call was slower than by the library's
+// transforms from 12 stacks of 64^2 and 4 of 128^2 on.  Images of 512^2 and
+// more have rows enough (and spill with two sets).
+template <int kLog, typename T> __host__ __device__ constexpr int fft_adjoint_groups() {
+  return sizeof(T) == 4 && kLog <= 8 ? 8 : 1;
+}
 template <typename T, typename C, int kLog>
-__global__ void __launch_bounds__(fft_row_threads<kLog>(), (sizeof(T) == 4 ? 384 : 256) / fft_row_threads<kLog>())
+__global__ void __launch_bounds__(fft_row_threads<kLog>() * fft_adjoint_groups<kLog, T>(),
+                                  fft_adjoint_groups<kLog, T>() > 1
+                                      ? 1
+                                      : (sizeof(T) == 4 ? 384 : 256) / fft_row_threads<kLog>())
     fft_rows_adjoint_kernel(const C* __restrict__ grids,
                             const typename PixelPhase<T>::omn* __restrict__ omn,
                             const T* __restrict__ corr, const double* __restrict__ wbar,
@@ -586,19 +600,25 @@ __global__ void __launch_bounds__(fft_row_threads<kLog>(), (sizeof(T) == 4 ? 384
                             const C* __restrict__ tab, T* __restrict__ x, int accumulate) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   struct __align__(2 * sizeof(C)) Pair { C c[2]; };
-  constexpr int N = 1 << kLog, TPR = N / 16;
-  const int j = threadIdx.x % TPR, rl = threadIdx.x / TPR;
-  C* sh = reinterpret_cast<C*>(smem_raw) + rl * fft_row_elems<kLog>();
+  constexpr int N = 1 << kLog, TPR = N / 16, kThreads = fft_row_threads<kLog>();
+  constexpr bool kSplit = fft_adjoint_groups<kLog, T>() > 1;
+  const int groups = kSplit ? static_cast<int>(blockDim.x) / kThreads : 1;
+  const int group = kSplit ? static_cast<int>(threadIdx.x) / kThreads : 0;
+  const int t = kSplit ? static_cast<int>(threadIdx.x) % kThreads : static_cast<int>(threadIdx.x);
+  const int j = t % TPR, rl = t / TPR;
+  C* sh = reinterpret_cast<C*>(smem_raw) + (group * fft_rows<kLog>() + rl) * fft_row_elems<kLog>();
   const int row = blockIdx.x * fft_rows<kLog>() + rl;
   const int64_t pix = static_cast<int64_t>(row) * N;
   T acc[16];
 #pragma unroll
   for (int m = 0; m < 16; ++m) acc[m] = T(0);
 #pragma unroll 1
-  for (int sl = 0; sl < nslots; ++sl) {
-    const PixelPhase<T> phase(wbar[stacks[sl]]);
+  for (int s0 = 0; s0 < nslots; s0 += groups) {
+    const int sl = s0 + group;
+    const bool on = !kSplit || sl < nslots;   // the others keep step at the block's barriers
+    const PixelPhase<T> phase(wbar[stacks[on ? sl : 0]]);
     const Pair* src = reinterpret_cast<const Pair*>(
-        grids + (static_cast<int64_t>(sl) * 2 * N + row) * 2 * N);
+        grids + (static_cast<int64_t>(on ? sl : 0) * 2 * N + row) * 2 * N);
     C even[16], odd[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
@@ -608,18 +628,39 @@ __global__ void __launch_bounds__(fft_row_threads<kLog>(), (sizeof(T) == 4 ? 384
     }
     fft_points<kLog, 1>(even, sh, j, tab);
     fft_points<kLog, 1>(odd, sh, j, tab);
+    if (on) {
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      const int n = j + m * TPR;
-      const C g = fft_add(even[m], fft_mul(odd[m], fft_root<1>(tab[n < N / 2 ? n : n + N])));
-      const C e = phase(omn[pix + (n ^ (N / 2))]);
-      acc[m] += e.x * g.x + e.y * g.y;
+      for (int m = 0; m < 16; ++m) {
+        const int n = j + m * TPR;
+        const C g = fft_add(even[m], fft_mul(odd[m], fft_root<1>(tab[n < N / 2 ? n : n + N])));
+        const C e = phase(omn[pix + (n ^ (N / 2))]);
+        acc[m] += e.x * g.x + e.y * g.y;
+      }
     }
   }
-#pragma unroll
-  for (int m = 0; m < 16; ++m) {
+  auto put = [&](int m, T sum) {
     const int64_t at = pix + ((j + m * TPR) ^ (N / 2));
-    const T v = corr[at] * acc[m];
+    const T v = corr[at] * sum;
     x[at] = accumulate ? x[at] + v : v;
+  };
+  if (!kSplit || groups == 1) {
+#pragma unroll
+    for (int m = 0; m < 16; ++m) put(m, acc[m]);
+    return;
   }
+  // [set][m][thread], over the exchange; the first set adds and stores (all
+  // sixteen loads of corr at once; a few m to each set, in turn, took 2 us more)
+  T* part = reinterpret_cast<T*>(smem_raw);
+  static_assert(16 * kThreads * sizeof(T) <= sizeof(C) * fft_rows<kLog>() * fft_row_elems<kLog>(),
+                "a set's sums must fit its exchange memory");
+  __syncthreads();
+#pragma unroll
+  for (int m = 0; m < 16; ++m) part[(group * 16 + m) * kThreads + t] = acc[m];
+  __syncthreads();
+  if (group) return;
+  for (int g = 1; g < groups; ++g)
+#pragma unroll
+    for (int m = 0; m < 16; ++m) acc[m] += part[(g * 16 + m) * kThreads + t];
+#pragma unroll
+  for (int m = 0; m < 16; ++m) put(m, acc[m]);
 }

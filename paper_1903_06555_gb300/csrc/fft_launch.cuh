@@ -84,10 +84,17 @@ int fft_pass_log(Plan& p, FftPass pass, const int32_t* stacks, int n, const T* x
           <<<cols(fft_cols_adjoint_kernel<T, C, kLog>), col_threads, col_smem, s>>>(
               tab, p.fft_maps, grids, tiles, p.fft_wait_limit, timeout);
       break;
-    case kFftRowsAdjoint:
-      fft_rows_adjoint_kernel<T, C, kLog><<<rows.y, row_threads, row_smem, s>>>(
+    case kFftRowsAdjoint: {
+      // sets of threads for the stacks while the sets of all blocks fit the
+      // chip at once (12 warps per SM of 170 registers)
+      int groups = 1;
+      while (2 * groups <= fft_adjoint_groups<kLog, T>() && groups < n &&
+             2 * groups * rows.y * (row_threads / 32) <= static_cast<unsigned>(12 * p.num_sms))
+        groups *= 2;
+      fft_rows_adjoint_kernel<T, C, kLog><<<rows.y, groups * row_threads, groups * row_smem, s>>>(
           grids, omn, corr, p.wbar_dev, stacks, n, tab, x_out, accumulate);
       break;
+    }
   }
   PHI_CUDA_TRY(cudaGetLastError());
   return PHI_OK;
@@ -114,7 +121,8 @@ int fft_setup_log(Plan& p) {
   const int row = static_cast<int>(sizeof(C) * fft_rows<kLog>() * fft_row_elems<kLog>());
   const int col = static_cast<int>(fft_col_smem<T, C, kLog>());
   PHI_CUDA_TRY(cudaFuncSetAttribute(fft_rows_forward_kernel<T, C, kLog>, a, row));
-  PHI_CUDA_TRY(cudaFuncSetAttribute(fft_rows_adjoint_kernel<T, C, kLog>, a, row));
+  PHI_CUDA_TRY(cudaFuncSetAttribute(fft_rows_adjoint_kernel<T, C, kLog>, a,
+                                    fft_adjoint_groups<kLog, T>() * row));
   PHI_CUDA_TRY(cudaFuncSetAttribute(fft_cols_forward_kernel<T, C, kLog>, a, col));
   PHI_CUDA_TRY(cudaFuncSetAttribute(fft_cols_adjoint_kernel<T, C, kLog>, a, col));
   return fft_make_maps_log<T, C, kLog>(p);

@@ -51,3 +51,12 @@ def grid_mib(n, precision):
 @pytest.mark.parametrize("precision", ["f32", "f64"])
 def test_groups_of_two_and_one(n, precision):
     check(n, 3, precision, 2, max(1, math.ceil(2 * grid_mib(n, precision))))
+
+
+# 64^2: eight grids of FP32 to a MiB
+@pytest.mark.parametrize("n,k,group,mib", [
+    (64, 9, 5, 1), (64, 20, 7, 1),           # groups of 5 + 4, and of 7 + 7 + 6
+    (64, 2, 2, 0), (64, 3, 3, 0), (64, 8, 8, 0), (64, 13, 13, 0), (64, 40, 40, 0),
+    (128, 2, 2, 0), (128, 24, 24, 0), (256, 5, 5, 0), (256, 20, 10, 20)])
+def test_small_images_with_many_stacks(n, k, group, mib):
+    check(n, k, "f32", group, mib)
