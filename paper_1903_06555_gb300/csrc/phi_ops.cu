@@ -409,15 +409,18 @@ int launch_pixel_tables(Plan& p, cudaStream_t s) {
 // S~_k then Z for every stack of a group (blockIdx.y = slot): grid cell
 // (qv, qu) holds padded pixel P = (q + Npad/2) mod Npad (the centred image
 // moved to index 0), i.e. image pixel P - (Npad - N)/2, or zero outside.
-// Npad is even: a thread writes two neighbouring cells in one store.  Bound:
-// the grid's bytes (with FP64 phases the FP64 unit was).
+// FP32 (Npad is even): a thread writes two neighbouring cells in one store.
+// Bound: the grid's bytes (with FP64 phases the FP64 unit was); FP64 its
+// FP64 unit, which two cells to a thread keep less evenly busy (240^2, 24
+// stacks: 125 us against 99).
 template <typename T, typename C>
 __global__ void prep_kernel(const T* __restrict__ x,
                             const typename PixelPhase<T>::omn* __restrict__ omn,
                             const T* __restrict__ corr, int N, int npad,
                             const double* __restrict__ wbar, const int32_t* __restrict__ stacks,
                             C* __restrict__ grids) {
-  struct __align__(2 * sizeof(C)) Pair { C c[2]; };
+  constexpr int kCells = sizeof(T) == 4 ? 2 : 1;
+  struct __align__(kCells * sizeof(C)) Cells { C c[kCells]; };
   const int off = (npad - N) / 2;
   const PixelPhase<T> phase(wbar[stacks[blockIdx.y]]);
   C* grid = grids + static_cast<int64_t>(blockIdx.y) * npad * npad;
@@ -426,10 +429,10 @@ __global__ void prep_kernel(const T* __restrict__ x,
     if (pv >= npad) pv -= npad;
     pv -= off;
     const bool row_in = pv >= 0 && pv < N;
-    for (int q0 = 2 * threadIdx.x; q0 < npad; q0 += 2 * blockDim.x) {
-      Pair out;
+    for (int q0 = kCells * threadIdx.x; q0 < npad; q0 += kCells * blockDim.x) {
+      Cells out;
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
+      for (int k = 0; k < kCells; ++k) {
         int pu = q0 + k + npad / 2;
         if (pu >= npad) pu -= npad;
         pu -= off;
@@ -442,7 +445,7 @@ __global__ void prep_kernel(const T* __restrict__ x,
           out.c[k].y = v * e.y;
         }
       }
-      *reinterpret_cast<Pair*>(grid + static_cast<int64_t>(qv) * npad + q0) = out;
+      *reinterpret_cast<Cells*>(grid + static_cast<int64_t>(qv) * npad + q0) = out;
     }
   }
 }
@@ -2240,7 +2243,12 @@ int image_to_grids(Plan& p, int g, int n, const T* x, C* grids, cudaStream_t s) 
   if (own_transform(p)) {
     PHI_TRY_ST((own_pass<T, C>(p, kFftRowsForward, stacks, n, x, grids, nullptr, 0, s)));
   } else {
-    prep_kernel<T, C><<<dim3(p.num_sms * 4, n), 256, 0, s>>>(
+    // no blocks without a row; narrow grids in FP32, two cells to a thread, in
+    // smaller blocks (100 stacks of 70^2: 72 us with neither, 31 with the
+    // first, 18 with both; of 240^2 104, 93, 52; from 1000^2 on 256 threads
+    // are the faster: one stack of 1988^2 39 and 50 us)
+    const int threads = sizeof(T) == 4 && p.npad <= 1280 ? 128 : 256;
+    prep_kernel<T, C><<<dim3(std::min(p.num_sms * 4, p.npad), n), threads, 0, s>>>(
         x, static_cast<const typename PixelPhase<T>::omn*>(p.omn_pix),
         static_cast<const T*>(p.corr_pix), p.N, p.npad, p.wbar_dev, stacks, grids);
     PHI_CUDA_TRY(cudaGetLastError());

@@ -60,3 +60,11 @@ def test_groups_of_two_and_one(n, precision):
     (128, 2, 2, 0), (128, 24, 24, 0), (256, 5, 5, 0), (256, 20, 10, 20)])
 def test_small_images_with_many_stacks(n, k, group, mib):
     check(n, k, "f32", group, mib)
+
+
+@pytest.mark.parametrize("n,k", [(70, 24), (640, 3), (642, 3)])
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+def test_blocks_of_the_image_step(n, k, precision):
+    """Grids narrower and wider than the image step's change of block (FP32,
+    Npad 1280), and fewer rows than it launches blocks for large ones."""
+    check(n, k, precision, k, 0)
