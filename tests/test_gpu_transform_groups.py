@@ -68,3 +68,21 @@ def test_blocks_of_the_image_step(n, k, precision):
     """Grids narrower and wider than the image step's change of block (FP32,
     Npad 1280), and fewer rows than it launches blocks for large ones."""
     check(n, k, precision, k, 0)
+
+
+def test_library_batches_with_a_grid_left_over():
+    """35 grids of 2000^2 exceed one batch of at most 1 GiB: two batches of 17
+    and one grid by itself, against the same stacks one grid at a time."""
+    geo = O.Geometry(1000, 2.0, math.radians(15.0), 4.0)
+    k = 35
+    uvw = W.uvw_disk(8 * k, 0.45 * geo.Npad * geo.du, 5.0 * k, 7)
+    x, yr = W.random_image(1000, 1), W.random_vis(len(uvw), 2)
+    got = []
+    for mib, group in ((0, k), (1, 1)):
+        plan = gpu_plan(uvw, geo, k, True, "f32", max_grid_mib=mib, max_support=128)
+        assert plan.info()["group"] == group
+        got.append((plan.degrid(to_t(x, torch.float32)).cpu().numpy(),
+                    plan.grid(to_t(yr, torch.complex64)).cpu().numpy()))
+        plan.close()
+    for a, b in zip(*got):
+        assert np.isfinite(a).all() and O.rel_l2(a, b) < 2e-6
