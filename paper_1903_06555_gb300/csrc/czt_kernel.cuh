@@ -251,8 +251,14 @@ __global__ void __launch_bounds__(czt_col_threads<kLog>())
   }
 }
 
+// As fft_rows_adjoint_kernel, the stacks over two sets of threads where the
+// rows of M = 1024 (380 to 512 pixels) fill a third of the chip: 50 stacks of
+// 394^2 440 us with one set, 292 with two (the whole call 1031 and 885, by the
+// library's transforms 1006); 24 of 498^2 264 and 188.
+template <int kLog> __host__ __device__ constexpr int czt_adjoint_groups() { return kLog == 10 ? 2 : 1; }
 template <int kLog>
-__global__ void __launch_bounds__(fft_row_threads<kLog>(), 512 / fft_row_threads<kLog>())
+__global__ void __launch_bounds__(fft_row_threads<kLog>() * czt_adjoint_groups<kLog>(),
+                                  512 / (fft_row_threads<kLog>() * czt_adjoint_groups<kLog>()))
     czt_rows_adjoint_kernel(const float2* __restrict__ grids,
                             const typename PixelPhase<float>::omn* __restrict__ omn,
                             const float* __restrict__ corr, const double* __restrict__ wbar,
@@ -260,36 +266,51 @@ __global__ void __launch_bounds__(fft_row_threads<kLog>(), 512 / fft_row_threads
                             const float2* __restrict__ tab, int N, float* __restrict__ x,
                             int accumulate) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int TPM = 1 << (kLog - 4);
+  constexpr int TPM = 1 << (kLog - 4), kThreads = fft_row_threads<kLog>();
+  constexpr bool kSplit = czt_adjoint_groups<kLog>() > 1;
+  static_assert(fft_rows<kLog>() == 1 && czt_adjoint_groups<kLog>() <= 2, "one row, two sets at most");
   const float2* c = tab + czt_roots(kLog);
-  const int j = threadIdx.x % TPM, rl = threadIdx.x / TPM;
-  float2* sh = reinterpret_cast<float2*>(smem_raw) + rl * fft_row_elems<kLog>();
-  const int row = blockIdx.x * fft_rows<kLog>() + rl;
+  const int groups = kSplit ? blockDim.x / kThreads : 1;
+  const int group = kSplit ? threadIdx.x / kThreads : 0, j = threadIdx.x % kThreads;
+  float2* sh = reinterpret_cast<float2*>(smem_raw) + group * fft_row_elems<kLog>();
+  const int row = blockIdx.x;
   float acc[8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) acc[m] = 0.0f;
 #pragma unroll 1
-  for (int sl = 0; sl < nslots; ++sl) {
-    const PixelPhase<float> phase(wbar[stacks[sl]]);
-    const float2* src = grids + (static_cast<int64_t>(sl) * 2 * N + row) * 2 * N;
+  for (int s0 = 0; s0 < nslots; s0 += groups) {
+    const int sl = s0 + group;
+    const bool on = !kSplit || sl < nslots;   // the other set keeps step at the barriers
+    const PixelPhase<float> phase(wbar[stacks[on ? sl : 0]]);
+    const float2* src = grids + (static_cast<int64_t>(on ? sl : 0) * 2 * N + row) * 2 * N;
     float2 out[8];
     czt_adjoint<kLog>(
-        out,
-        [&](int parity, int n) { return row < N ? src[2 * n + parity] : make_float2(0.0f, 0.0f); },
-        c, N, sh, j, tab, c + 2 * N);
+        out, [&](int parity, int n) { return src[2 * n + parity]; }, c, N, sh, j, tab, c + 2 * N);
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       const int n = j + m * TPM;
-      if (n < N && row < N) {
+      if (n < N && on) {
         const float2 e = phase(omn[static_cast<int64_t>(row) * N + (n < N / 2 ? n + N / 2 : n - N / 2)]);
         acc[m] += e.x * out[m].x + e.y * out[m].y;
       }
     }
   }
+  if (kSplit && groups > 1) {   // the second set's sums, over the exchange
+    float* part = reinterpret_cast<float*>(smem_raw);
+    __syncthreads();
+    if (group) {
+#pragma unroll
+      for (int m = 0; m < 8; ++m) part[m * kThreads + j] = acc[m];
+    }
+    __syncthreads();
+    if (group) return;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) acc[m] += part[m * kThreads + j];
+  }
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
     const int n = j + m * TPM;
-    if (n < N && row < N) {
+    if (n < N) {
       const int64_t at = static_cast<int64_t>(row) * N + (n < N / 2 ? n + N / 2 : n - N / 2);
       const float v = corr[at] * acc[m];
       x[at] = accumulate ? x[at] + v : v;

@@ -26,10 +26,12 @@ int czt_pass_log(Plan& p, FftPass pass, const int32_t* stacks, int n, const floa
     case kFftColsAdjoint:
       czt_cols_adjoint_kernel<kLog><<<cols, col_threads, col_smem, s>>>(tab, N, grids);
       break;
-    case kFftRowsAdjoint:
-      czt_rows_adjoint_kernel<kLog><<<rows.y, row_threads, row_smem, s>>>(
+    case kFftRowsAdjoint: {
+      const int groups = std::min(n, czt_adjoint_groups<kLog>());
+      czt_rows_adjoint_kernel<kLog><<<rows.y, groups * row_threads, groups * row_smem, s>>>(
           grids, omn, corr, p.wbar_dev, stacks, n, tab, N, x_out, accumulate);
       break;
+    }
   }
   PHI_CUDA_TRY(cudaGetLastError());
   return PHI_OK;
