@@ -476,8 +476,9 @@ __host__ __device__ inline int dde_series_bytes(int jmax, int jd) {
   return 2 * jd * 16 + static_cast<int>(sizeof(C)) *
                            (kDdeRows * (jmax + 2 * h2) + (kDdeRows + h2) * (jmax + h2));
 }
-// kJd: the DDE's taps a side when known at compile time (0: any).
-template <typename T, typename C, bool kGrid, int kJd>
+// kJd: the DDE's taps a side when known at compile time (0: any).  kAgain as
+// in series_take.
+template <typename T, typename C, bool kGrid, int kJd, bool kAgain>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) dde_series_kernel(
     const VisRec<T>* __restrict__ recs, const uint32_t* __restrict__ perm, int64_t n,
     const C* __restrict__ grid_in, C* grid_out, const C* __restrict__ vis_in,
@@ -503,8 +504,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) dde_series_kernel
   WarpQueue wq;
   unsigned long long i0;
   int nv, pass, P;
-  while (series_take<T, C>(w, wq, head, static_cast<unsigned long long>(batch), n, recs, sv, q,
-                           lane, i0, nv, pass, P)) {
+  while (series_take<kAgain, T, C>(w, wq, head, static_cast<unsigned long long>(batch), n, recs, sv, q,
+                           lane, i0, nv, pass, P, my_nodes)) {
 #pragma unroll 1
     for (int v = 0; v < nv; ++v) {
       if (!((pass >> v) & 1)) continue;
@@ -608,7 +609,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) dde_series_kernel
         for (int cu = lane; cu < Jc; cu += 32)
           for (int row = 0; row < h2; ++row) R[row * rw + cu] = R[(row + kDdeRows) * rw + cu];
       }
-      if (lane == 0) my_nodes += static_cast<unsigned long long>((NP + 1) * kNodes * P);
+      if (!kAgain && lane == 0)
+        my_nodes += static_cast<unsigned long long>((NP + 1) * kNodes * P);
       if (!kGrid) store_visibility<T, C>(accv, static_cast<T>(r.weight), pm, vis_out, lane);
       __syncwarp();   // the polynomials, the band and R are rewritten
     }

@@ -119,10 +119,12 @@ int launch_dde_series(Plan& p, int g, const VisRec<T>* recs, int64_t b0, int64_t
   const int jmax = std::max(p.max_jw, 2);
   const size_t extra = static_cast<size_t>(dde_series_bytes<C>(jmax, dde.jd));
   // the usual small kernels unrolled, any other in a loop
-  auto kernel = dde.jd == 3   ? dde_series_kernel<T, C, kGrid, 3>
-                : dde.jd == 5 ? dde_series_kernel<T, C, kGrid, 5>
-                : dde.jd == 7 ? dde_series_kernel<T, C, kGrid, 7>
-                              : dde_series_kernel<T, C, kGrid, 0>;
+  constexpr bool f64 = sizeof(T) == 8;
+  auto kernel = !f64 && p.series_again ? dde_series_kernel<T, C, kGrid, 0, true>
+                : dde.jd == 3          ? dde_series_kernel<T, C, kGrid, 3, f64>
+                : dde.jd == 5          ? dde_series_kernel<T, C, kGrid, 5, f64>
+                : dde.jd == 7          ? dde_series_kernel<T, C, kGrid, 7, f64>
+                                       : dde_series_kernel<T, C, kGrid, 0, f64>;
   SeriesShape sh;
   PHI_TRY_ST((series_shape<T, C>(p, kernel, nk, extra, sh)));
   launched = sh.warps > 0;

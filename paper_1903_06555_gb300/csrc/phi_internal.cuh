@@ -252,6 +252,7 @@ struct Plan {
   float4* series_nodes = nullptr;
   uint32_t* retry = nullptr;
   int series_stride = 0, series_max_panels = 0, series_max_intervals = 0;
+  bool series_again = false;   // tables with a panel more, for visibilities that fail the estimate
   float series_inv_cycles = 0;
   // deterministic gridding (grid_deterministic = 1): fixed-point sums of the
   // group's grids (group * Npad^2 * 2 int64), the largest |W_i y_i| term

@@ -2464,23 +2464,32 @@ void timer_end(Plan& p, long idx, int stage, cudaStream_t s) {
   p.ev_pending.emplace_back(stage, static_cast<size_t>(idx));
 }
 
-template <typename T, typename C, int kJd>
+template <typename T, typename C, int kJd, bool kAgain>
 cudaError_t set_dde_series_smem(int bytes) {
   const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(dde_series_kernel<T, C, false, kJd>, a, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(dde_series_kernel<T, C, true, kJd>, a, bytes);
+  cudaError_t e = cudaFuncSetAttribute(dde_series_kernel<T, C, false, kJd, kAgain>, a, bytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(dde_series_kernel<T, C, true, kJd, kAgain>, a, bytes);
+  return e;
+}
+template <typename T, typename C, bool kAgain>
+cudaError_t set_vis_series_smem(int bytes) {
+  const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(vis_series_kernel<T, C, false, kAgain>, a, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(vis_series_kernel<T, C, true, kAgain>, a, bytes);
   return e;
 }
 
 template <typename T, typename C>
 cudaError_t set_series_smem(int bytes) {
-  const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(vis_series_kernel<T, C, false>, a, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(vis_series_kernel<T, C, true>, a, bytes);
-  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 0>(bytes);
-  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 3>(bytes);
-  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 5>(bytes);
-  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 7>(bytes);
+  constexpr bool f64 = sizeof(T) == 8;   // which has no kernels without kAgain
+  cudaError_t e = set_vis_series_smem<T, C, true>(bytes);
+  if (e == cudaSuccess) e = set_vis_series_smem<T, C, f64>(bytes);
+  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 0, true>(bytes);
+  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 0, f64>(bytes);
+  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 3, f64>(bytes);
+  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 5, f64>(bytes);
+  if (e == cudaSuccess) e = set_dde_series_smem<T, C, 7, f64>(bytes);
   return e;
 }
 

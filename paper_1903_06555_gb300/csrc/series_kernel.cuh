@@ -197,10 +197,10 @@ __device__ __forceinline__ SeriesB series_split(const float (&v)[4]) {
 // real or imaginary part; a visibility that is not there has dw = 0 and is
 // ignored) into smp (visibility v at smp + v * vstride, its first samples also
 // mirrored to negative rho).  Returns whether the estimate passes at this
-// lane's samples 0 .. NP of visibility t = lane % 4, NP that visibility's.  Every
-// column is computed alike, so a visibility's samples do not depend on what
-// it is sampled with.
-template <int MT>
+// lane's samples 0 .. NP of visibility t = lane % 4, NP that visibility's (-1:
+// it keeps the samples it has).  Every column is computed alike, so a
+// visibility's samples do not depend on what it is sampled with.
+template <int MT, bool kAgain>
 __device__ __forceinline__ bool series_sample_f32(float2* smp, int vstride,
                                                   const SeriesView<float>& sv, int P,
                                                   const PhaseF& phase, int m0, int NP, int lane) {
@@ -264,8 +264,10 @@ __device__ __forceinline__ bool series_sample_f32(float2* smp, int vstride,
     for (int i = 0; i < 2; ++i) {
       const int s = kSeriesTile * (m0 + m) + g + 8 * i;
       const float2 k = make_float2(kUnscale * K[m][2 * i], kUnscale * K[m][2 * i + 1]);
-      smp[s] = k;
-      if (m == 0 && m0 == 0 && s < SeriesN<float>::half) smp[-s] = k;   // even in rho
+      if (!kAgain || NP >= 0) {
+        smp[s] = k;
+        if (m == 0 && m0 == 0 && s < SeriesN<float>::half) smp[-s] = k;   // even in rho
+      }
       if (s <= NP) good = good && 1.5f * kUnscale * err[m][i] <= sv.tol;   // NaN fails
     }
   return good;
@@ -498,8 +500,10 @@ struct SeriesWarp {
 };
 
 // Samples of the taken visibilities (the lane's dw: FP32 the one of its B
-// column, FP64 the visibility's; NP: intervals of visibility lane % 4, top:
-// the most of any); bit v of the result: visibility v passes.
+// column, FP64 the visibility's; NP: intervals of visibility lane % 4, or -1
+// for one that keeps the samples it has, top: the most of any); bit v of the
+// result: visibility v passes.
+template <bool kAgain>
 __device__ __forceinline__ int series_sample(SeriesWarp<float, float2>& w,
                                              const SeriesView<float>& sv, const QuadParams&,
                                              int P, double dw, int NP, int top, int lane) {
@@ -508,15 +512,15 @@ __device__ __forceinline__ int series_sample(SeriesWarp<float, float2>& w,
   bool good = true;
   int m0 = 0;
   for (; tiles > 4; tiles -= 4, m0 += 4)
-    good = series_sample_f32<4>(w.smp, w.vstride, sv, P, phase, m0, NP, lane) && good;
+    good = series_sample_f32<4, kAgain>(w.smp, w.vstride, sv, P, phase, m0, NP, lane) && good;
   if (tiles == 4)
-    good = series_sample_f32<4>(w.smp, w.vstride, sv, P, phase, m0, NP, lane) && good;
+    good = series_sample_f32<4, kAgain>(w.smp, w.vstride, sv, P, phase, m0, NP, lane) && good;
   else if (tiles == 3)
-    good = series_sample_f32<3>(w.smp, w.vstride, sv, P, phase, m0, NP, lane) && good;
+    good = series_sample_f32<3, kAgain>(w.smp, w.vstride, sv, P, phase, m0, NP, lane) && good;
   else if (tiles == 2)
-    good = series_sample_f32<2>(w.smp, w.vstride, sv, P, phase, m0, NP, lane) && good;
+    good = series_sample_f32<2, kAgain>(w.smp, w.vstride, sv, P, phase, m0, NP, lane) && good;
   else
-    good = series_sample_f32<1>(w.smp, w.vstride, sv, P, phase, m0, NP, lane) && good;
+    good = series_sample_f32<1, kAgain>(w.smp, w.vstride, sv, P, phase, m0, NP, lane) && good;
   const unsigned bad = __ballot_sync(0xffffffffu, !good);
   __syncwarp();
   int pass = 0;
@@ -524,6 +528,7 @@ __device__ __forceinline__ int series_sample(SeriesWarp<float, float2>& w,
   for (int v = 0; v < 4; ++v) pass |= (bad & (0x11111111u << v)) ? 0 : 1 << v;
   return pass;
 }
+template <bool kAgain>
 __device__ __forceinline__ int series_sample(SeriesWarp<double, double2>& w,
                                              const SeriesView<double>& sv, const QuadParams& q,
                                              int P, double dw, int NP, int, int lane) {
@@ -544,13 +549,22 @@ __device__ __forceinline__ int series_sample(SeriesWarp<double, double2>& w,
 // the same panels behind it in this batch; samples them, and puts those that
 // fail on the retry list.  A visibility beyond the tables goes to the list
 // at once.  False at the end.
-template <typename T, typename C>
+//
+// kAgain: one whose estimate fails is first sampled again on one panel more, if
+// the tables go so far.  At some supports every visibility fails on the
+// a-priori panels: where the taper is narrow against the first of them (12
+// pixels of support, J_w 14, one panel of 5.4 cycles: 1.5 E = 8e-6).  One panel
+// more brings E down by two orders and more; the list would take the whole
+// observation (20,000 such visibilities: 212 us by the list, 72 sampled again;
+// the per-tap kernel by itself 195).  FP32 plans without such supports take
+// the kernels without it (its registers spill, 1% of the snapshot's time).
+template <bool kAgain, typename T, typename C>
 __device__ __forceinline__ bool series_take(SeriesWarp<T, C>& w, WarpQueue& wq,
                                             unsigned long long* head, unsigned long long batch,
                                             int64_t n, const VisRec<T>* __restrict__ recs,
                                             const SeriesView<T>& sv, const QuadParams& q,
                                             int lane, unsigned long long& i0, int& nv, int& pass,
-                                            int& P) {
+                                            int& P, unsigned long long& nodes) {
   constexpr int NV = SeriesVis<T>::n;
   while (wq.take(head, batch, n, lane, i0)) {
     // the lane's candidate: FP32 the visibility of its B column
@@ -574,8 +588,21 @@ __device__ __forceinline__ bool series_take(SeriesWarp<T, C>& w, WarpQueue& wq,
     const int own = v < nv ? myNP : 0;
     const int top = __reduce_max_sync(0xffffffffu, own);
     // intervals of the visibility whose sums this lane will hold
-    const int NP = __shfl_sync(0xffffffffu, own, NV > 1 ? 8 * (lane & 3) : 0);
-    pass = series_sample(w, sv, q, P, v < nv ? dw : 0.0, NP, top, lane);
+    int NP = __shfl_sync(0xffffffffu, own, NV > 1 ? 8 * (lane & 3) : 0);
+    if constexpr (kAgain) {
+      pass = 0;
+#pragma unroll 1
+      for (int p = P, last = min(P + 1, sv.max_panels);; ++p) {
+        // evaluations, counted by one lane of each visibility's columns
+        if (v < nv && (lane & (NV > 1 ? 7 : 31)) == 0 && !((pass >> v) & 1))
+          nodes += (myNP + 1) * kNodes * p;
+        pass |= series_sample<kAgain>(w, sv, q, p, v < nv ? dw : 0.0, NP, top, lane);
+        if (p >= last || !(~pass & ((1 << nv) - 1))) break;
+        if (NV > 1 && ((pass >> (lane & 3)) & 1)) NP = -1;
+      }
+    } else {   // counted with the taps
+      pass = series_sample<kAgain>(w, sv, q, P, v < nv ? dw : 0.0, NP, top, lane);
+    }
     if (lane < nv && !((pass >> lane) & 1))
       sv.retry[atomicAdd(sv.n_retry, 1ULL)] = static_cast<uint32_t>(i0) + lane;
     return true;
@@ -674,7 +701,7 @@ __device__ __forceinline__ void series_taps(const SeriesWarp<double, double2>& w
 
 // Degrid / grid of visibilities [0, n): one warp per visibility (sampling
 // four at a time in FP32), taken from the work queue.
-template <typename T, typename C, bool kGrid>
+template <typename T, typename C, bool kGrid, bool kAgain>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
     vis_series_kernel(const VisRec<T>* __restrict__ recs, const uint32_t* __restrict__ perm,
                       int64_t n, const C* __restrict__ grid_in, C* grid_out,
@@ -690,8 +717,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
   WarpQueue wq;
   unsigned long long i0;
   int nv, pass, P;
-  while (series_take<T, C>(w, wq, head, static_cast<unsigned long long>(batch), n, recs, sv, q,
-                           lane, i0, nv, pass, P)) {
+  while (series_take<kAgain, T, C>(w, wq, head, static_cast<unsigned long long>(batch), n, recs,
+                                   sv, q, lane, i0, nv, pass, P, my_nodes)) {
 #pragma unroll 1
     for (int v = 0; v < nv; ++v) {
       if (!((pass >> v) & 1)) continue;
@@ -722,7 +749,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
       }
       if (lane == 0) {
         my_taps += static_cast<unsigned long long>(rv.jw * rv.jw);
-        my_nodes += static_cast<unsigned long long>((NP + 1) * kNodes * P);
+        if (!kAgain) my_nodes += static_cast<unsigned long long>((NP + 1) * kNodes * P);
       }
       if (!kGrid) store_visibility<T, C>(acc, static_cast<T>(rv.weight), pm, vis_out, lane);
       __syncwarp();   // the polynomials are rewritten for the next visibility

@@ -28,6 +28,28 @@ SeriesView<T> series_view(const Plan& p, int g) {
 template <typename T>
 constexpr double series_least_tol() { return sizeof(T) == 4 ? 2.5e-7 : 1e-14; }
 
+// Whether visibilities of supports up to jw may fail on their a-priori panels.
+// Evaluated in 64 bits for supports J of 2 to 64 pixels, oversampling 1.25 to
+// 3, windows of 0.25 to 1 cycles, offsets from 0 to those of J_w up to J + 60
+// and tolerances from these limits to 1e-6 (FP64 1e-12), those that do have
+// few panels for their J, nearly filled: at most J / 4 panels in FP32 (1 below
+// 8) and J / 2 in FP64, of 0.7 of the a-priori width and more (FP32, J <= 4:
+// 0.87; FP64 0.6, but for J = 2 at 1e-14).  With one panel more all but one of
+// 28,000 combinations pass.
+template <typename T>
+bool series_may_fail(const Plan& p, int jw) {
+  const bool f64 = sizeof(T) == 8;
+  const int J = p.d.support, most = f64 ? std::max(2, J / 2) : std::max(1, J / 4);
+  const double least = f64 ? 0.6 : J <= 4 ? 0.85 : 0.7;
+  for (int w = J; w <= jw; w += 2) {
+    const double want = p.R * (w * 0.70710678 + 0.5 * (w - J)) * p.series_inv_cycles;
+    const double n = std::max(1.0, std::ceil(want));
+    if (n > most) break;
+    if (want > least * n) return true;
+  }
+  return false;
+}
+
 // J0 table for the panel counts and supports of this plan.  Panels no wider
 // than the automatic width, so that a plan with wide panels of its own still
 // passes the estimate.
@@ -45,6 +67,8 @@ int build_series_tables_t(Plan& p, cudaStream_t s) {
                                             static_cast<float>(p.c_support), p.series_inv_cycles,
                                             static_cast<float>(p.stack_maxabs[k])));
   }
+  p.series_again = series_may_fail<T>(p, p.max_jw);
+  if (p.series_again) ++panels;
   p.series_max_panels = std::min(panels, kSeriesMaxPanels);
   p.series_max_intervals = std::min(intervals, kSeriesMaxSamples - SeriesN<T>::half);
   const int grain = sizeof(T) == 4 ? kSeriesTile : 32;   // samples of a tile, of a warp
@@ -133,9 +157,12 @@ template <typename T, typename C, bool kGrid>
 int launch_series(Plan& p, int g, const VisRec<T>* recs, int64_t b0, int64_t nk, const C* grids_in,
                   C* grids_out, const C* vis_in, C* vis_out, cudaStream_t s) {
   SeriesShape sh;
-  PHI_TRY_ST((series_shape<T, C>(p, vis_series_kernel<T, C, kGrid>, nk, 0, sh)));
+  constexpr bool f64 = sizeof(T) == 8;
+  auto kernel = p.series_again ? vis_series_kernel<T, C, kGrid, true>
+                               : vis_series_kernel<T, C, kGrid, f64>;
+  PHI_TRY_ST((series_shape<T, C>(p, kernel, nk, 0, sh)));
   if (sh.warps == 0) return PHI_ERR_SUPPORT;   // not reached: one warp takes 31 KB at most
-  vis_series_kernel<T, C, kGrid><<<sh.blocks, 32 * sh.warps, sh.smem, s>>>(
+  kernel<<<sh.blocks, 32 * sh.warps, sh.smem, s>>>(
       recs, p.perm + b0, nk, grids_in, grids_out, vis_in, vis_out, p.quad(),
       series_view<T, C>(p, g), p.stack_slot_dev, p.counters + g, p.counters + p.K, sh.batch);
   PHI_CUDA_TRY(cudaGetLastError());
