@@ -34,7 +34,7 @@
 // (gathered from one table of W^k they took 16 wavefronts a load).
 #pragma once
 
-constexpr int kFftMinLog = 6, kFftMaxLog = 11;
+constexpr int kFftMinLog = 6, kFftMinLog64 = 9, kFftMaxLog = 11;
 
 // log2 N when the two-pass transforms take the plan's grid, or 0.  FP64 from
 // N = 512 on (six stacks of 512^2: 0.76 ms, separate steps 1.11); below, its
@@ -42,7 +42,7 @@ constexpr int kFftMinLog = 6, kFftMaxLog = 11;
 // 0.050 ms).
 __host__ inline int fft_log(int N, int npad, bool f64) {
   if (npad != 2 * N) return 0;
-  for (int l = f64 ? 9 : kFftMinLog; l <= kFftMaxLog; ++l)
+  for (int l = f64 ? kFftMinLog64 : kFftMinLog; l <= kFftMaxLog; ++l)
     if (N == 1 << l) return l;
   return 0;
 }

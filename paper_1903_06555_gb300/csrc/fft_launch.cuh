@@ -100,17 +100,30 @@ int fft_pass_log(Plan& p, FftPass pass, const int32_t* stacks, int n, const T* x
   return PHI_OK;
 }
 
+// call(log2 N as a constant) for the plan's size: 2^6 .. 2^11 in FP32, 2^9 ..
+// 2^11 in FP64 (fft_log).
+template <typename T, typename F>
+int fft_dispatch(const Plan& p, F call) {
+  if constexpr (sizeof(T) == 4) {
+    switch (p.fft_log) {
+      case 6: return call(std::integral_constant<int, 6>());
+      case 7: return call(std::integral_constant<int, 7>());
+      case 8: return call(std::integral_constant<int, 8>());
+    }
+  }
+  switch (p.fft_log) {
+    case 9: return call(std::integral_constant<int, 9>());
+    case 10: return call(std::integral_constant<int, 10>());
+    default: return call(std::integral_constant<int, 11>());
+  }
+}
+
 template <typename T, typename C>
 int fft_pass(Plan& p, FftPass pass, const int32_t* stacks, int n, const T* x_in, C* grids,
              T* x_out, int accumulate, cudaStream_t s) {
-  switch (p.fft_log) {
-    case 6: return fft_pass_log<T, C, 6>(p, pass, stacks, n, x_in, grids, x_out, accumulate, s);
-    case 7: return fft_pass_log<T, C, 7>(p, pass, stacks, n, x_in, grids, x_out, accumulate, s);
-    case 8: return fft_pass_log<T, C, 8>(p, pass, stacks, n, x_in, grids, x_out, accumulate, s);
-    case 9: return fft_pass_log<T, C, 9>(p, pass, stacks, n, x_in, grids, x_out, accumulate, s);
-    case 10: return fft_pass_log<T, C, 10>(p, pass, stacks, n, x_in, grids, x_out, accumulate, s);
-    default: return fft_pass_log<T, C, 11>(p, pass, stacks, n, x_in, grids, x_out, accumulate, s);
-  }
+  return fft_dispatch<T>(p, [&](auto log) {
+    return fft_pass_log<T, C, log.value>(p, pass, stacks, n, x_in, grids, x_out, accumulate, s);
+  });
 }
 
 // Dynamic shared memory limits (fixed per kernel, the same for every plan) and
@@ -129,12 +142,5 @@ int fft_setup_log(Plan& p) {
 }
 template <typename T, typename C>
 int fft_setup(Plan& p) {
-  switch (p.fft_log) {
-    case 6: return fft_setup_log<T, C, 6>(p);
-    case 7: return fft_setup_log<T, C, 7>(p);
-    case 8: return fft_setup_log<T, C, 8>(p);
-    case 9: return fft_setup_log<T, C, 9>(p);
-    case 10: return fft_setup_log<T, C, 10>(p);
-    default: return fft_setup_log<T, C, 11>(p);
-  }
+  return fft_dispatch<T>(p, [&](auto log) { return fft_setup_log<T, C, log.value>(p); });
 }
