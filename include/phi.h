@@ -45,10 +45,11 @@
  *     modes the sums over them, and the estimate, are formed at samples of
  *     rho at twice the rate the kernel's band limit asks for, and every tap
  *     is interpolated from them (to FP32 and FP64 rounding); a visibility
- *     whose samples show that each of its taps meets quad_abs_tol is done,
- *     any other one is integrated tap by tap (quadrature) or from its
- *     Chebyshev series (radial), as all are when quad_abs_tol is below
- *     2.5e-7 in FP32 or 1e-14 in FP64.  Taps that do not converge within the
+ *     whose estimate is at most quad_abs_tol / 1.5 at every sample within its
+ *     box is done, any other one is sampled once more on one panel more or
+ *     integrated tap by tap (quadrature) or from its Chebyshev series
+ *     (radial), as all are when quad_abs_tol is below 2.5e-7 in FP32 or 1e-14
+ *     in FP64.  Taps that do not converge within the
  *     refinement cap are counted (phi_plan_stats), never an error.
  *
  * Memory and streams: every pointer argument named *_dev is a device pointer
@@ -94,7 +95,10 @@ enum phi_status {
 
 enum phi_precision {
   PHI_F32 = 0,  /* FP32 grid, FFT, kernel, accumulation and quadrature error
-                   estimate; chirp phases in pairs of FP32 values            */
+                   estimate; chirp phases in pairs of FP32 values (48 bits),
+                   the factors of the sampled quadrature's node sums in pairs
+                   of FP16 values (22 bits, the products of the low halves
+                   left out) summed in FP32                                  */
   PHI_F64 = 1   /* everything in FP64                                        */
 };
 

@@ -14,7 +14,9 @@
 // first 8 of 16 values.
 //
 // Bound: the exchanges through shared memory, like fft_kernel.cuh's, at four
-// times the length per point: 8 grids of 3972^2, forward 2.94 ms, adjoint 3.11
+// times the length per point, and spills: czt_forward holds the input, both
+// halves of the output and the 16 working values (152 to 432 bytes a thread at
+// 128 registers; the adjoint, which takes the halves in turn, 4 to 152): 8 grids of 3972^2, forward 2.94 ms, adjoint 3.11
 // (image steps and cuFFT 5.62 and 5.50), 3.4e-7 and 3.2e-7 from 64 bits (5.2e-7
 // and 4.6e-7).
 #pragma once

@@ -14,8 +14,8 @@
 // integrand, h(r_j) = 2 pi h_p g(r_j) r_j e^{-2 pi i dw (n(r_j) - 1)}, is the
 // same for all J_w^2 taps of the visibility, so the lanes first build it at
 // the Gauss-Kronrod 15/31 nodes of an a-priori partition of [0, R] into
-// equal panels (tabulated 1 - n(r_j) and g(r_j); FP32 forms the phase in two
-// floats), then each lane takes two taps and sums J0(2 pi rho r_j) h(r_j) with the Kronrod
+// equal panels (FP64 phase argument, tabulated 1 - n(r_j) and g(r_j)), then
+// each lane takes two taps and sums J0(2 pi rho r_j) h(r_j) with the Kronrod
 // weights, and, per panel, the difference against the embedded Gauss rule
 // as the error estimate (FP32 path: in paired f32x2 arithmetic, two nodes
 // per instruction).  A chunk of 64 taps whose estimate misses
@@ -589,7 +589,7 @@ __global__ void fixed_to_grid_kernel(const longlong2* __restrict__ cells,
 
 // Build the weighted integrand values for panels [p0, p0 + np) of the
 // npan-panel partition: h(r_j) e^{2 pi i dw (1 - n(r_j))}, phase argument in
-// FP64 or two floats, one NodeVal per node (FP64 path: Kronrod and difference weights).
+// FP64, one NodeVal per node (FP64 path: Kronrod and difference weights).
 template <typename T>
 __device__ __forceinline__ void build_nodes(NodeVal<T>* sh, const QuadParams& q, int npan, int p0,
                                             int np, double dw, int lane) {

@@ -17,17 +17,26 @@
 // 10) products and a short polynomial per tap in place of 31 P J_w^2 Bessel
 // functions.
 //
-// Tolerance.  The estimate E = sum over panels |K31 - G15| is formed at every
-// sample.  Each panel's difference is band-limited like the kernel, and a
-// function sampled at twice its Nyquist rate is bounded between the samples
-// by 1 / cos(pi / 4) = 1.42 times its largest sample, so a visibility whose
-// samples satisfy 1.5 E <= quad_abs_tol has every tap within the tolerance.
+// Tolerance.  The estimate E = sum over panels |K31 - G15| is formed at the
+// samples within the box, and a visibility is settled if 1.5 E <= quad_abs_tol
+// at all of them.  That is an estimate of the taps' E, as G15 against K31 is
+// one of their error, not a bound: were the samples of the whole line tested,
+// no tap's E could exceed 1 / cos(pi / 4) = 1.42 times the largest (each
+// panel's difference is band-limited like the kernel and sampled at twice its
+// Nyquist rate; one sum of the panels with the phases that align them at the
+// tap is too), but those beyond the box, which the interpolation reads (9; FP64
+// 19) and the panels are not sized for, are not.  Of 3,400 random supports,
+// windows, oversamplings, offsets and tolerances whose samples passed,
+// evaluated in 64 bits, no tap's E exceeded 0.63 of the tolerance.  The taps'
+// values do not depend on it: the sums over the nodes are band-limited by
+// construction, whatever their error against the integral.
 // The a-priori panels follow the support (the corner of the box and the
 // largest |dw| the support covers), which leaves E two orders below 1e-6 at
-// 6 cycles per panel.  A visibility that fails -- or needs more panels or
-// samples than the tables hold -- is put on a list, and the kernel that
-// integrates each tap by itself (vis_kernel and its companions), with its
-// refinement and its count of unconverged taps, takes that list.
+// 6 cycles per panel for the default support.  A visibility that fails -- or
+// needs more panels or samples than the tables hold -- is put on a list, and
+// the kernel that integrates each tap by itself (vis_kernel and its
+// companions), with its refinement and its count of unconverged taps, takes
+// that list.
 //
 // FP32 makes the sums on the tensor cores (series_tile_kernel says how the
 // operands are split), four visibilities of one panel count to a warp: 1.3 ms
