@@ -1,12 +1,13 @@
 """Benchmark: w-corrected visibilities/s (degrid + grid) of the GB300
 w-stacking w-projection operator on the MWA-like snapshot workload
 (2048^2 image, 4096^2 grid, FOV 25 deg, 1.95M visibilities, 8 k-means
-w-stacks, conjugate fold, FP32 with FP64 chirp phase, quadrature tol 1e-6).
+w-stacks, conjugate fold, FP32 with chirp phases in pairs of FP32 values,
+quadrature tol 1e-6).
 
 One step = one y = Phi x (phi_degrid) plus one x = Re(Phi^H y) (phi_grid)
 over every visibility, i.e. every stage of the hot path: per stack S~_k/Z,
-cuFFT, fused w-kernel quadrature + degridding, fused quadrature + gridding,
-inverse cuFFT, crop/chirp/sum.  The plan (fold, Algorithm 1, sort) is built
+transform, fused w-kernel quadrature + degridding, fused quadrature +
+gridding, inverse transform, crop/chirp/sum.  The plan (fold, Algorithm 1, sort) is built
 once per observation and timed separately; the e2e figure includes it.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
@@ -220,15 +221,17 @@ def kernel_source_hash():
     import hashlib
     h = hashlib.sha256()
     for f in ("phi_ops.cu", "bessel_j0.cuh", "phi_internal.cuh", "table_index.cuh",
-              "fixed_point.cuh", "series_kernel.cuh", "series_coef.cuh", "fft_kernel.cuh", "czt_kernel.cuh"):
+              "fixed_point.cuh", "series_kernel.cuh", "series_launch.cuh", "series_coef.cuh",
+              "fft_kernel.cuh", "fft_launch.cuh", "czt_kernel.cuh", "czt_launch.cuh"):
         with open(os.path.join(ROOT, "paper_1903_06555_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
 
 def profiled_traffic(stage):
-    """DRAM bytes per launch of the fused kernel from the committed ncu launch
-    list, or None when the kernel sources changed since it was taken."""
+    """DRAM bytes per launch of the fused kernel (degrid, grid; table_degrid,
+    table_grid with the w rows staged) from the committed ncu capture of the
+    full workload, or None when the kernel sources changed since it was taken."""
     p = os.path.join(ROOT, "profiles", "vis_series_kernel_mwa-2048.md")
     if not os.path.exists(p):
         return None
@@ -628,9 +631,8 @@ def run_ours(args, ws, rank, local):
         hbm_peak = peaks.get("hbm_gbs", 6800.0)
         roof["hbm"] = {"achieved_gbs": gbs, "peak_gbs": hbm_peak, "frac": gbs / hbm_peak}
 
-    # grids the library transforms by its own two-pass kernels
-    own_fft = info["npad"] == 2 * wl.image_n and wl.image_n in [2 ** k for k in
-                                                                range(9 if f64 else 6, 12)]
+    # grids the library transforms by its own kernels
+    own_fft = plan.transform() != "library"
 
     # end to end through the public API from pinned host buffers
     e2e = run_e2e(phi, desc, uvw_np, x_np, args.e2e_steps, dev) if args.e2e_steps > 0 else None
@@ -787,7 +789,8 @@ def run_e2e(phi, desc, uvw_np, x_np, steps, dev):
             "h2d_bytes_per_step": int(uvw_h.numel() * 8 + x_h.numel() * x_h.element_size()),
             "d2h_bytes_per_step": int(y_h.numel() * y_h.element_size() +
                                       d_h.numel() * d_h.element_size()),
-            "note": "includes plan build (fold, k-means, sort, tables, cuFFT plan)"}
+            "note": "includes plan build (fold, k-means, sort, tables of the quadrature and "
+                    "the transforms)"}
 
 
 # ---------------------------------------------------------------------------- serving

@@ -272,6 +272,14 @@ int phi_plan_info(phi_plan_t plan, phi_plan_summary* info, double* wbar, int64_t
 int phi_plan_stats(phi_plan_t plan, int64_t* n_unconverged, int64_t* n_taps,
                    int64_t* n_tap_nodes, int reset, void* stream);
 
+/* Which transforms the plan's grids take (enum phi_transform; -1 for NULL). */
+enum phi_transform {
+  PHI_TRANSFORM_LIBRARY = 0,   /* image step and cuFFT                        */
+  PHI_TRANSFORM_TWO_PASS = 1,  /* rows and columns, images of 2^6 to 2^11     */
+  PHI_TRANSFORM_CHIRP = 2      /* rows and columns, as convolutions           */
+};
+int phi_plan_transform(phi_plan_t plan);
+
 /* How often the column passes of this plan's transforms poll for a copy of
  * theirs before they give up (phi_plan_stats), about a microsecond a poll.
  * Plans start with 2^20, which polls < 0 or above restores; 0 makes every

@@ -34,6 +34,7 @@ PHI_SUPPORT_STACK, PHI_SUPPORT_VIS = 0, 1
 PHI_KERNEL_QUADRATURE, PHI_KERNEL_TABLE, PHI_KERNEL_RADIAL = 0, 1, 2
 STAGES = ("prep", "fft", "degrid", "grid", "finish", "clear")
 NUM_STAGES = len(STAGES)
+TRANSFORMS = ("library", "two-pass", "chirp")   # enum phi_transform
 
 
 class PlanDesc(ctypes.Structure):
@@ -139,6 +140,7 @@ def lib():
             L.phi_plan_info.argtypes = [_vp, ctypes.POINTER(PlanSummary), _vp, _vp, _vp]
             L.phi_plan_stats.argtypes = [_vp, ctypes.POINTER(_i64), ctypes.POINTER(_i64),
                                          ctypes.POINTER(_i64), ctypes.c_int, _vp]
+            L.phi_plan_transform.argtypes = [_vp]
             L.phi_plan_set_wait_limit.argtypes = [_vp, ctypes.c_int]
             L.phi_plan_set_timing.argtypes = [_vp, ctypes.c_int]
             L.phi_plan_timings.argtypes = [_vp, ctypes.POINTER(ctypes.c_double),
@@ -361,6 +363,10 @@ class Plan:
         _check(lib().phi_plan_stats(self._h, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c),
                                     int(reset), _stream(stream)), "phi_plan_stats")
         return int(a.value), int(b.value), int(c.value)
+
+    def transform(self) -> str:
+        """What transforms the plan's grids: 'library', 'two-pass' or 'chirp'."""
+        return TRANSFORMS[lib().phi_plan_transform(self._h)]
 
     def set_wait_limit(self, polls=-1):
         """Polls of a transform's wait before it gives up (-1: the default).

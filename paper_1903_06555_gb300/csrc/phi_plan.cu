@@ -1003,6 +1003,12 @@ extern "C" int phi_plan_stats(phi_plan_t plan, int64_t* n_unconverged, int64_t* 
   return h[4] ? PHI_ERR_TIMEOUT : PHI_OK;
 }
 
+extern "C" int phi_plan_transform(phi_plan_t plan) {
+  if (!plan) return -1;
+  return plan->fft_log ? PHI_TRANSFORM_TWO_PASS
+                       : plan->czt_log ? PHI_TRANSFORM_CHIRP : PHI_TRANSFORM_LIBRARY;
+}
+
 extern "C" int phi_plan_set_wait_limit(phi_plan_t plan, int polls) {
   if (!plan) return PHI_ERR_ARG;
   const int most = phi::transform_wait_limit();
