@@ -447,7 +447,9 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
                             int* __restrict__ timeout) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bar;
-  __shared__ int failed;   // a thread's wait ran out; read after the next barrier
+  // a thread's wait ran out, read after the next barrier (__syncthreads_or, as
+  // in the adjoint, spills here)
+  __shared__ int failed;
   constexpr int N = 1 << kLog, TPC = N / 16, NC = fft_cols<kLog, T>(), kTiles = 2 * N / NC;
   const int c = threadIdx.x % NC, j = threadIdx.x / NC;
   C* in = reinterpret_cast<C*>(fft_aligned(smem_raw));
@@ -513,7 +515,6 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
                             int* __restrict__ timeout) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bars[2];
-  __shared__ int failed;   // a thread's wait ran out; read after the next barrier
   constexpr int N = 1 << kLog, TPC = N / 16, NC = fft_cols<kLog, T>(), kTiles = 2 * N / NC;
   const int c = threadIdx.x % NC, j = threadIdx.x / NC;
   C* buf = reinterpret_cast<C*>(fft_aligned(smem_raw));   // even rows
@@ -522,7 +523,6 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
   C* sh = out + c * fft_col_elems<kLog, T>();
   const bool lead = threadIdx.x == 0;
   if (lead) {
-    failed = 0;
     fft_bar_init(&bars[0]);
     fft_bar_init(&bars[1]);
     const int col = blockIdx.x % kTiles * NC, grid = blockIdx.x / kTiles;
@@ -530,26 +530,39 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
     fft_tile_load<C, N, NC, true>(buf1, &maps, col, 1, grid, &bars[1]);
   }
   __syncthreads();
-  unsigned parity = 0, parity0 = 0;   // parity0: of the load last sent to the even rows' buffer
+  unsigned parity = 0;
   int tile = blockIdx.x;
+  // leaves; parity0: of the load last sent to the even rows' buffer (one load
+  // may be in flight to each)
+  auto give_up = [&](unsigned parity0) {
+    if (lead) {
+      fft_bar_wait(&bars[0], parity0, kFftWaitLimit);
+      fft_bar_wait(&bars[1], parity, kFftWaitLimit);
+    }
+    __syncthreads();
+    fft_give_up<T, C, N, NC>(grids, N, tile, tiles, timeout);
+  };
   for (; tile < tiles; tile += gridDim.x, parity ^= 1) {
     const int col = tile % kTiles * NC, grid = tile / kTiles, next = tile + gridDim.x;
     C even[16], v[16];
-    if (!fft_bar_wait(&bars[0], parity, limit)) failed = 1;
+    bool late = !fft_bar_wait(&bars[0], parity, limit);
 #pragma unroll
     for (int m = 0; m < 16; ++m) even[m] = buf[(j + m * TPC) * NC + c];
     if (lead) fft_stores_read();   // the exchange's memory is free again
-    __syncthreads();               // and the even rows have been read
-    if (failed) break;             // the whole block
-    parity0 = next < tiles ? parity ^ 1 : parity;
+    if (__syncthreads_or(late)) {  // and the even rows have been read
+      give_up(parity);             // the whole block
+      break;
+    }
     if (lead && next < tiles)
       fft_tile_load<C, N, NC, true>(buf, &maps, next % kTiles * NC, 0, next / kTiles, &bars[0]);
     fft_points<kLog, 1>(even, sh, j, tab);
-    if (!fft_bar_wait(&bars[1], parity, limit)) failed = 1;
+    late = !fft_bar_wait(&bars[1], parity, limit);
 #pragma unroll
     for (int m = 0; m < 16; ++m) v[m] = buf1[(j + m * TPC) * NC + c];
-    __syncthreads();               // the odd rows have been read
-    if (failed) break;             // the whole block
+    if (__syncthreads_or(late)) {  // the odd rows have been read
+      give_up(next < tiles ? parity ^ 1 : parity);
+      break;
+    }
     if (lead && next < tiles)
       fft_tile_load<C, N, NC, true>(buf1, &maps, next % kTiles * NC, 1, next / kTiles, &bars[1]);
     fft_points<kLog, 1>(v, sh, j, tab);
@@ -563,14 +576,6 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
     fft_publish();
     __syncthreads();
     if (lead) fft_tile_store<C, N, NC, false>(out, &maps, col, 0, grid);
-  }
-  if (failed) {   // one load may be in flight to each buffer
-    if (lead) {
-      fft_bar_wait(&bars[0], parity0, kFftWaitLimit);
-      fft_bar_wait(&bars[1], parity, kFftWaitLimit);
-    }
-    __syncthreads();
-    fft_give_up<T, C, N, NC>(grids, N, tile, tiles, timeout);
   }
   if (lead) fft_stores_done();
 }
@@ -588,11 +593,9 @@ __global__ void __launch_bounds__(fft_col_threads<kLog, T>())
 template <int kLog, typename T> __host__ __device__ constexpr int fft_adjoint_groups() {
   return sizeof(T) == 4 && kLog <= 8 ? 8 : 1;
 }
-template <typename T, typename C, int kLog>
-__global__ void __launch_bounds__(fft_row_threads<kLog>() * fft_adjoint_groups<kLog, T>(),
-                                  fft_adjoint_groups<kLog, T>() > 1
-                                      ? 1
-                                      : (sizeof(T) == 4 ? 384 : 256) / fft_row_threads<kLog>())
+template <typename T, typename C, int kLog, bool kSplit>
+__global__ void __launch_bounds__(fft_row_threads<kLog>() * (kSplit ? fft_adjoint_groups<kLog, T>() : 1),
+                                  kSplit ? 1 : (sizeof(T) == 4 ? 384 : 256) / fft_row_threads<kLog>())
     fft_rows_adjoint_kernel(const C* __restrict__ grids,
                             const typename PixelPhase<T>::omn* __restrict__ omn,
                             const T* __restrict__ corr, const double* __restrict__ wbar,
@@ -601,7 +604,6 @@ __global__ void __launch_bounds__(fft_row_threads<kLog>() * fft_adjoint_groups<k
   extern __shared__ __align__(16) unsigned char smem_raw[];
   struct __align__(2 * sizeof(C)) Pair { C c[2]; };
   constexpr int N = 1 << kLog, TPR = N / 16, kThreads = fft_row_threads<kLog>();
-  constexpr bool kSplit = fft_adjoint_groups<kLog, T>() > 1;
   const int groups = kSplit ? static_cast<int>(blockDim.x) / kThreads : 1;
   const int group = kSplit ? static_cast<int>(threadIdx.x) / kThreads : 0;
   const int t = kSplit ? static_cast<int>(threadIdx.x) % kThreads : static_cast<int>(threadIdx.x);
@@ -643,7 +645,7 @@ __global__ void __launch_bounds__(fft_row_threads<kLog>() * fft_adjoint_groups<k
     const T v = corr[at] * sum;
     x[at] = accumulate ? x[at] + v : v;
   };
-  if (!kSplit || groups == 1) {
+  if (!kSplit) {
 #pragma unroll
     for (int m = 0; m < 16; ++m) put(m, acc[m]);
     return;

@@ -91,7 +91,10 @@ int fft_pass_log(Plan& p, FftPass pass, const int32_t* stacks, int n, const T* x
       while (2 * groups <= fft_adjoint_groups<kLog, T>() && groups < n &&
              2 * groups * rows.y * (row_threads / 32) <= static_cast<unsigned>(12 * p.num_sms))
         groups *= 2;
-      fft_rows_adjoint_kernel<T, C, kLog><<<rows.y, groups * row_threads, groups * row_smem, s>>>(
+      constexpr bool split = fft_adjoint_groups<kLog, T>() > 1;
+      auto kernel = groups > 1 ? fft_rows_adjoint_kernel<T, C, kLog, split>
+                               : fft_rows_adjoint_kernel<T, C, kLog, false>;
+      kernel<<<rows.y, groups * row_threads, groups * row_smem, s>>>(
           grids, omn, corr, p.wbar_dev, stacks, n, tab, x_out, accumulate);
       break;
     }
@@ -134,8 +137,11 @@ int fft_setup_log(Plan& p) {
   const int row = static_cast<int>(sizeof(C) * fft_rows<kLog>() * fft_row_elems<kLog>());
   const int col = static_cast<int>(fft_col_smem<T, C, kLog>());
   PHI_CUDA_TRY(cudaFuncSetAttribute(fft_rows_forward_kernel<T, C, kLog>, a, row));
-  PHI_CUDA_TRY(cudaFuncSetAttribute(fft_rows_adjoint_kernel<T, C, kLog>, a,
-                                    fft_adjoint_groups<kLog, T>() * row));
+  constexpr int groups = fft_adjoint_groups<kLog, T>();
+  PHI_CUDA_TRY(cudaFuncSetAttribute(fft_rows_adjoint_kernel<T, C, kLog, false>, a, row));
+  if (groups > 1)
+    PHI_CUDA_TRY(cudaFuncSetAttribute(fft_rows_adjoint_kernel<T, C, kLog, (groups > 1)>, a,
+                                      groups * row));
   PHI_CUDA_TRY(cudaFuncSetAttribute(fft_cols_forward_kernel<T, C, kLog>, a, col));
   PHI_CUDA_TRY(cudaFuncSetAttribute(fft_cols_adjoint_kernel<T, C, kLog>, a, col));
   return fft_make_maps_log<T, C, kLog>(p);
